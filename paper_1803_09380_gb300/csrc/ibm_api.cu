@@ -265,6 +265,69 @@ void choose_ib_grid(Ctx& c) {
   c.ib_jc_cluster = c.ib_phases == 2 && M > kSmallIbMarkers ? jacobi_cluster_size(c.prec, M) : 0;
 }
 
+// Markers that one slice of the barrier-free correction owns when the caller
+// has not set a CTA count: an even share for every SM, between a smallest
+// slice (below it the neighbourhood outweighs what it saves) and the largest
+// that leaves room for the neighbourhood of ten iterations.
+int slice_size(const Ctx& c) {
+  const int lo = c.r_bytes == 8 ? 8 : 16;
+  return std::max(lo, std::min(128, (c.nm + c.ib_grid_max - 1) / c.ib_grid_max));
+}
+
+// Plans the barrier-free correction for the current band: builds the slices'
+// lists, halving the slices while one does not fit.  Without it (moving
+// bodies, another launch form asked for, markers too dense for any slice, no
+// memory) steps run the persistent kernel.  Synchronises the stream once
+// per attempt; a stream that is being captured is left alone.
+void plan_slices(Ctx& c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
+  c.sl_tried = true;
+  if (c.nm == 0 || c.any_moving || !c.band_collide || c.ib_phases != 0 || c.ib_threads != kIbThreads ||
+      c.test_drop_arrival || c.desc.n_corr < 1 || c.desc.n_corr > slice_max_corr())
+    return;
+  if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 4 * sizeof(int)))) return;
+  const int asked = c.ib_grid_opt > 0 ? (c.nm + c.ib_grid - 1) / c.ib_grid : 0;
+  for (int S = asked ? asked : slice_size(c); S >= 1; S /= 2) {
+    const int count = (c.nm + S - 1) / S;
+    if (count > kSliceMaxCount) break;
+    c.sl_S = S;
+    c.sl_count = count;
+    c.sl_mem = dev_alloc(c, slice_mem_bytes(c.prec, count));
+    if (!c.sl_mem) break;
+    int stat[4] = {0, 0, 0, 0};
+    cudaError_t e = cudaMemsetAsync(c.dslstat, 0, sizeof(stat), c.stream);
+    if (e == cudaSuccess) e = launch_slice_build(c, c.dslstat, c.stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(stat, c.dslstat, sizeof(stat), cudaMemcpyDeviceToHost, c.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
+    if (e == cudaSuccess && stat[0] == 0) {
+      c.sl_xmax = (stat[1] + 31) / 32 * 32;
+      c.sl_x1max = (stat[2] + 31) / 32 * 32;
+      if (slice_smem(c.prec, c.desc.n_corr, c.sl_xmax, c.sl_x1max) > 0) {
+        c.sl_on = true;
+        return;
+      }
+    }
+    dev_free(c, c.sl_mem);
+    c.sl_mem = nullptr;
+    if (e != cudaSuccess) { cudaGetLastError(); break; }
+    if (asked) break;
+  }
+  c.sl_count = 0;
+}
+
+// Forgets the slices (the band, or an option that they depend on, changes);
+// the caller has synchronised the stream and drops the graphs.
+void drop_slices(Ctx& c) {
+  if (c.sl_mem) dev_free(c, c.sl_mem);
+  c.sl_mem = nullptr;
+  c.sl_on = c.sl_tried = false;
+  c.sl_count = 0;
+}
+
 ibm_status upload_markers(Ctx* h) {
   Ctx& c = *h;
   const int M = c.nm;
@@ -278,6 +341,7 @@ ibm_status upload_markers(Ctx* h) {
   IBM_CK(h, cudaMemsetAsync(c.dsegflag, 0, sizeof(int) * (size_t)c.nseg_x * c.geom.ny, c.stream));
   IBM_CK(h, cudaMemsetAsync(c.dctr, 0, CTR_COUNT * sizeof(int), c.stream));
   IBM_CK(h, cudaStreamSynchronize(c.stream));
+  drop_slices(c);
   dev_free(c, c.dseglist);
   c.dseglist = nullptr;
   for (void* p : olds) dev_free(c, p);
@@ -697,6 +761,7 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
         if (st != IBM_OK) return st;
       }
     }
+    if (c.nm > 0 && !c.sl_tried) plan_slices(c);
     const bool want_macro = !(flags & IBM_STEP_NO_MACRO);
     for (int k = 0; k < nsteps;) {
       const int parity = c.parity;
@@ -1061,6 +1126,7 @@ ibm_status ibm_set_option(ibm_handle h, int option, long long value) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     h->ib_threads = (int)value;
     h->ib_cluster_max = -1;
+    drop_slices(*h);
     choose_ib_grid(*h);
     destroy_graphs(*h);
     return IBM_OK;
@@ -1070,6 +1136,7 @@ ibm_status ibm_set_option(ibm_handle h, int option, long long value) {
     DeviceGuard guard(h->device);
     if (h->stream) cudaStreamSynchronize(h->stream);
     h->ib_phases = (int)value;
+    drop_slices(*h);
     choose_ib_grid(*h);
     destroy_graphs(*h);
     if (h->ib_phases == 1 && h->band_valid) return count_band(h);
@@ -1090,6 +1157,7 @@ ibm_status ibm_set_option(ibm_handle h, int option, long long value) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     if (option == IBM_OPT_BARRIER_LIMIT_US) h->bar_limit_ns = value * 1000LL;
     else h->test_drop_arrival = (int)value;
+    drop_slices(*h);
     destroy_graphs(*h);                  // the kernels take both as arguments
     return IBM_OK;
   }
@@ -1098,6 +1166,7 @@ ibm_status ibm_set_option(ibm_handle h, int option, long long value) {
   h->ib_grid_opt = (int)value;
   DeviceGuard guard(h->device);
   if (h->stream) cudaStreamSynchronize(h->stream);
+  drop_slices(*h);
   choose_ib_grid(*h);
   destroy_graphs(*h);
   return IBM_OK;

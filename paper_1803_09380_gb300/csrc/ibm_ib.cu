@@ -522,6 +522,10 @@ static void ib_loop_t(const Ctx& h, int parity, bool macro, cudaStream_t s) {
 }
 
 void launch_ib_loop(const Ctx& h, int parity, bool macro, cudaStream_t s) {
+  if (h.sl_on) {
+    launch_slice_loop(h, parity, macro, s);
+    return;
+  }
   switch (h.prec) {
     case PREC_FP64: ib_loop_t<PREC_FP64>(h, parity, macro, s); break;
     case PREC_FP32: ib_loop_t<PREC_FP32>(h, parity, macro, s); break;

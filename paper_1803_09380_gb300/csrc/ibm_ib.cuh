@@ -540,6 +540,55 @@ __device__ __forceinline__ void deviation(const Args& a, int l, const R* __restr
   djx = a.mq[4 * l + 1] - sx;
   djy = a.mq[4 * l + 2] - sy;
 }
+// Eq. 29: partial force and torque of each body over one fixed chunk of
+// kForceChunk markers (one CTA), F_l = -ds_l A^N_l, T_l = (X_l - x_c) x F_l,
+// FP64; the chunking does not depend on the grid, so neither do the sums.
+template <int P, int NT>
+__device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typename Prec<P>::R* __restrict__ AN, int k,
+                                               double* sh) {
+  if (a.nb <= 0) return;
+  const int lo = k * kForceChunk, hi = min(a.M, lo + kForceChunk);
+  const int b0 = a.mbody[lo], b1 = a.mbody[hi - 1];
+  for (int bd = b0; bd <= b1; ++bd) {
+    const BodyDev& B = a.bodies[bd];
+    const int l0 = max(lo, B.m0), l1 = min(hi, B.m1);
+    double fx = 0.0, fy = 0.0, tq = 0.0;
+    for (int l = l0 + (int)threadIdx.x; l < l1; l += NT) {
+      const double Fx = -a.ds[l] * (double)AN[2 * l], Fy = -a.ds[l] * (double)AN[2 * l + 1];
+      fx += Fx;
+      fy += Fy;
+      tq += (a.X[l] - B.xc[0]) * Fy - (a.Y[l] - B.xc[1]) * Fx;
+    }
+    block_sum3(fx, fy, tq, sh);
+    if (threadIdx.x == 0) {
+      double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
+      o[0] = fx; o[1] = fy; o[2] = tq;
+    }
+  }
+}
+
+// Body totals: bodies rank, rank + nranks, .. by this CTA, fixed-shape
+// reduction over the chunks (which other CTAs may have written in this
+// launch: read past the L1 cache).
+template <int P, int NT>
+__device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks, double* sh) {
+  for (int bd = rank; bd < a.nb; bd += nranks) {
+    BodyDev& B = a.bodies[bd];
+    const int k0 = B.m0 / kForceChunk, k1 = (B.m1 - 1) / kForceChunk;
+    double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+    for (int k = k0 + (int)threadIdx.x; k <= k1; k += NT) {
+      const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
+      f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
+    }
+    block_sum3(f0, f1, f2, sh);
+    if (threadIdx.x == 0) {
+      B.F_ib[0] = f0;
+      B.F_ib[1] = f1;
+      B.T_ib = f2;
+    }
+  }
+}
+
 // The correction loop of one step in phases.  Each phase runs on nth
 // threads numbered tid (band-node work from the other end, rtid = nth - 1 -
 // tid), grouped in CTAs of NT threads numbered rank of nranks; a phase reads
@@ -712,33 +761,7 @@ __device__ __forceinline__ void ib_phase_final(const IbArgs<P>& a, int tid, int 
       a.bq[8 * b + 7] = dy;
     }
   }
-  // Eq. 29: partial force and torque of each body over fixed chunks of
-  // kForceChunk markers (CTAs take chunks in turn), F_l = -ds_l A^N_l,
-  // T_l = (X_l - x_c) x F_l, FP64; the chunking does not depend on the grid,
-  // so neither do the sums.
-  const int nchunk = (M + kForceChunk - 1) / kForceChunk;
-  if (a.nb > 0) {
-    for (int k = rank; k < nchunk; k += nranks) {
-      const int lo = k * kForceChunk, hi = min(M, lo + kForceChunk);
-      const int b0 = a.mbody[lo], b1 = a.mbody[hi - 1];
-      for (int bd = b0; bd <= b1; ++bd) {
-        const BodyDev& B = a.bodies[bd];
-        const int l0 = max(lo, B.m0), l1 = min(hi, B.m1);
-        double fx = 0.0, fy = 0.0, tq = 0.0;
-        for (int l = l0 + (int)threadIdx.x; l < l1; l += NT) {
-          const double Fx = -a.ds[l] * (double)AN[2 * l], Fy = -a.ds[l] * (double)AN[2 * l + 1];
-          fx += Fx;
-          fy += Fy;
-          tq += (a.X[l] - B.xc[0]) * Fy - (a.Y[l] - B.xc[1]) * Fx;
-        }
-        block_sum3(fx, fy, tq, sh);
-        if (threadIdx.x == 0) {
-          double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
-          o[0] = fx; o[1] = fy; o[2] = tq;
-        }
-      }
-    }
-  }
+  for (int k = rank; k < (M + kForceChunk - 1) / kForceChunk; k += nranks) ib_force_chunk<P, NT>(a, AN, k, sh);
 }
 
 // r^N is complete: a non-finite residual means the state has diverged; one
@@ -783,23 +806,7 @@ __device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, in
     }
   }
 
-  // body totals: one body per CTA, fixed-shape reduction over the chunks
-  for (int bd = rank; bd < a.nb; bd += nranks) {
-    BodyDev& B = a.bodies[bd];
-    const int k0 = B.m0 / kForceChunk, k1 = (B.m1 - 1) / kForceChunk;
-    double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-    for (int k = k0 + (int)threadIdx.x; k <= k1; k += NT) {
-      const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
-      f0 += o[0]; f1 += o[1]; f2 += o[2];
-    }
-    block_sum3(f0, f1, f2, sh);
-    if (threadIdx.x == 0) {
-      B.F_ib[0] = f0;
-      B.F_ib[1] = f1;
-      B.T_ib = f2;
-    }
-  }
-
+  ib_force_total<P, NT>(a, rank, nranks, sh);
 }
 
 // Folds the CTA's warp maxima in red[] into *dst (integer maximum of the

@@ -132,6 +132,13 @@ struct Ctx {
                                              // kernels, 2 Jacobi iterations in one cluster
   int ib_jc_cluster = 0;                     // CTAs of that cluster (0: not available)
   long long nband_host = 0;                  // band nodes at the last count (sizes the phase grids)
+  // barrier-free correction (ibm_slice.cuh): the slices of the current band
+  bool sl_tried = false;                     // planned for the current band and options
+  bool sl_on = false;                        // steps run on the slices
+  int sl_count = 0, sl_S = 0;                // slices, markers owned by each
+  int sl_xmax = 0, sl_x1max = 0;             // largest local node counts
+  void* sl_mem = nullptr;                    // the slices' lists
+  int* dslstat = nullptr;                    // [4] build status
   long long watch_due = 0;                   // steps since the last watchdog scan
 
   // CUDA graphs of one step, per parity and macro flag
@@ -212,6 +219,23 @@ inline void launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStr
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = 0;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributePriority;
+  attr[0].val.priority = prio;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// The same launch with dynamic shared memory.
+template <typename... KArgs, typename... Args>
+inline void launch_prio_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int prio,
+                             Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributePriority;
@@ -302,6 +326,17 @@ constexpr int kMaxIbCluster = 16;
 // CTAs of the cluster that runs the Jacobi iterations of M markers (0: none).
 int jacobi_cluster_size(int prec, int M);
 void launch_body_update(const Ctx& h, cudaStream_t s);
+
+// ibm_slice.cu: the barrier-free correction loop
+constexpr int kSliceMaxCount = 2048;
+size_t slice_mem_bytes(int prec, int count);
+// Builds the lists of h.sl_count slices of h.sl_S markers into h.sl_mem;
+// stat (device, 3 ints, zeroed): a slice did not fit, largest node counts.
+cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s);
+// Dynamic shared memory of the slice kernel (0: it does not fit).
+size_t slice_smem(int prec, int N, int xmax, int x1max);
+int slice_max_corr();
+void launch_slice_loop(const Ctx& h, int parity, bool macro, cudaStream_t s);
 // Rigid motion of every moving body's markers to its current pose (Eqs. 41-42).
 void launch_marker_move(const Ctx& h, cudaStream_t s);
 

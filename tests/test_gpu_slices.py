@@ -1,0 +1,114 @@
+"""The barrier-free correction (each CTA iterates its slice of markers with
+the neighbourhood it depends on) against the launch form with one kernel per
+phase: the same arithmetic per element in the same order, so every result is
+bitwise the same, whatever the slices."""
+import math
+
+import numpy as np
+import pytest
+
+from _helpers import gpu_lattice
+from paper_1803_09380_gb300 import ibm
+from paper_1803_09380_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _rings(n, radii, spacing=1.0, at=None, **kw):
+    """Fixed rings of the given radii around one point, turning alternately."""
+    bodies = []
+    for k, r in enumerate(radii):
+        m = max(3, int(round(2 * math.pi * r / spacing)))
+        c = (n / 2.0 + 0.3, n / 2.0 - 0.2) if at is None else at[k]
+        xy, ds = wl.ring(c[0], c[1], r, count=m)
+        bodies.append(wl.Body(xy, ds, wl.BODY_FIXED, xc=c, omega=0.01 / r * (-1) ** k, radius=r))
+    return wl.Case("rings", n, n, 0.8, bodies=bodies, **kw)
+
+
+CASES = {
+    # two rings of 878 markers, the default slices; one slice; many
+    "couette256": lambda: wl.couette(256),
+    # rings 1.5 apart: every marker couples with both rings
+    "near": lambda: _rings(96, (20.0, 21.5)),
+    # a ring across the periodic edges
+    "edge": lambda: _rings(64, (17.0,), at=[(1.2, 62.9)]),
+    # half a unit apart (rows of about twenty), and markers that share no node
+    "dense": lambda: _rings(96, (30.0,), spacing=0.5),
+    "sparse": lambda: _rings(96, (40.0,), spacing=5.0),
+    # a single marker; a bare triangle
+    "one": lambda: wl.Case("one", 32, 32, 0.8, bodies=[
+        wl.Body(np.array([[15.3, 16.6]]), np.ones(1), wl.BODY_FIXED, xc=(15.3, 16.6), u=(0.01, 0.005))]),
+    "three": lambda: _rings(32, (2.0,), spacing=4.0),
+    # closed and open sides, odd sizes; the lattice's last rows and columns in the supports
+    "box": lambda: _rings(61, (27.9,), at=[(30.0, 30.0)], bc=(wl.BOUNCEBACK,) * 4, wall_u=(0,) * 6 + (0.03, 0)),
+    "channel": lambda: wl.cylinder(nx=161, ny=77, diameter=20.0, center=(40.2, 38.1), markers=63),
+    "channel_nee": lambda: wl.paper_cylinder(40.0, diameter=12),
+    # other delta functions and iteration counts
+    "delta2": lambda: _delta(2),
+    "delta3": lambda: _delta(3),
+    "n1": lambda: _rings(128, (25.0, 50.0), n_corr=1),
+    "n2": lambda: _rings(128, (25.0, 50.0), n_corr=2),
+    "n25": lambda: _rings(128, (25.0, 50.0), n_corr=25),
+}
+
+
+def _delta(points):
+    c = _rings(96, (30.0,))
+    c.delta_points = points
+    return c
+
+
+def _run(case, prec, steps, phases=0, ctas=0):
+    lat = gpu_lattice(case, prec)
+    rho, ux, uy = wl.random_fields(case.nx, case.ny, 5, du=0.01, drho=0.001)
+    lat.init_equilibrium(rho, ux, uy)
+    if phases:
+        ibm.ibm_set_option(lat.h, ibm.IBM_OPT_IB_PHASES, phases)
+    if ctas:
+        lat.set_ib_ctas(ctas)
+    lat.step(steps)
+    out = (lat.f, lat.resid, lat.bodies, *lat.moments())
+    lat.close()
+    return out
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_slices_are_bitwise_the_phase_kernels(name, prec):
+    case = CASES[name]()
+    ref = _run(case, prec, 11, phases=1)
+    assert np.all(np.isfinite(ref[0]))
+    for got, want in zip(_run(case, prec, 11), ref):
+        assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("ctas", [4, 7, 33, 152])
+def test_slice_sizes_do_not_change_results(ctas):
+    """878 markers in 4 slices (220 of a CTA's 256 local markers are owned:
+    they do not fit, the persistent kernel runs), 7, 33 and 147."""
+    case = wl.couette(256)
+    ref = _run(case, "fp32", 9, phases=1)
+    for got, want in zip(_run(case, "fp32", 9, ctas=ctas), ref):
+        assert np.array_equal(got, want)
+
+
+def test_slices_follow_added_bodies_and_marker_velocities():
+    """Adding a body and prescribing velocities between steps: the slices are
+    rebuilt for the new band."""
+    out = []
+    for phases in (0, 1):
+        case = _rings(128, (25.0, 50.0))
+        lat = ibm.Lattice(case.nx, case.ny, case.tau, prec="fp32")
+        if phases:
+            ibm.ibm_set_option(lat.h, ibm.IBM_OPT_IB_PHASES, phases)
+        for b in case.bodies:
+            lat.add_markers(b.xy, b.ds, **b.as_kwargs())
+            lat.step(5)
+        m = sum(len(b.xy) for b in case.bodies)
+        uv = 0.01 * np.random.default_rng(3).standard_normal((m, 2))
+        lat.set_marker_velocities(uv)
+        lat.step(4)
+        out.append((lat.f, lat.resid, lat.bodies))
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
