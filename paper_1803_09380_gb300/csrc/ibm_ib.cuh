@@ -457,22 +457,31 @@ __device__ __forceinline__ void warp_max_to(R v, R* red) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
 }
 
-// Block sums of three doubles with a fixed-shape reduction (warp butterfly,
-// then the warp totals in warp order).
-__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, double* sh) {
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, off);
-    b += __shfl_xor_sync(0xffffffffu, b, off);
-    c += __shfl_xor_sync(0xffffffffu, c, off);
-  }
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if ((threadIdx.x & 31) == 0) { sh[w] = a; sh[32 + w] = b; sh[64 + w] = c; }
+// Sums of three doubles over the CTA's first kForceChunk threads, complete in
+// thread 0; the tree's shape does not depend on the CTA's size.  FP64 adds
+// issue at two lanes a clock on an SM, so the halving tree (24 warp-wide
+// adds) is taken instead of a butterfly in every warp (60 and more).
+__device__ __forceinline__ void chunk_sum3(double& a, double& b, double& c, double* sh) {
+  static_assert(kForceChunk == 128, "the tree below adds 128 values");
+  const int t = threadIdx.x;
+  if (t >= 64 && t < 128) { sh[t - 64] = a; sh[t] = b; sh[64 + t] = c; }
   __syncthreads();
-  a = sh[0]; b = sh[32]; c = sh[64];
-  for (int k = 1; k < nw; ++k) { a += sh[k]; b += sh[32 + k]; c += sh[64 + k]; }
+  if (t < 64) { a += sh[t]; b += sh[64 + t]; c += sh[128 + t]; }
+  __syncthreads();
+  if (t >= 32 && t < 64) { sh[t - 32] = a; sh[t] = b; sh[32 + t] = c; }
+  __syncthreads();
+  if (t < 32) {
+    a += sh[t]; b += sh[32 + t]; c += sh[64 + t];
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, off);
+      b += __shfl_down_sync(0xffffffffu, b, off);
+      c += __shfl_down_sync(0xffffffffu, c, off);
+    }
+  }
   __syncthreads();
 }
+constexpr int kChunkSumShared = 192;                 // doubles of shared memory it uses
 
 template <class R> struct Vec2;
 template <> struct Vec2<float> { typedef float2 T; };
@@ -541,46 +550,56 @@ __device__ __forceinline__ void deviation(const Args& a, int l, const R* __restr
   djy = a.mq[4 * l + 2] - sy;
 }
 // Eq. 29: partial force and torque of each body over one fixed chunk of
-// kForceChunk markers (one CTA), F_l = -ds_l A^N_l, T_l = (X_l - x_c) x F_l,
-// FP64; the chunking does not depend on the grid, so neither do the sums.
-template <int P, int NT>
+// kForceChunk markers (one CTA, a marker per thread), F_l = -ds_l A^N_l,
+// T_l = (X_l - x_c) x F_l, FP64; the chunking does not depend on the grid, so
+// neither do the sums.
+template <int P>
 __device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typename Prec<P>::R* __restrict__ AN, int k,
                                                double* sh) {
   if (a.nb <= 0) return;
+  __shared__ int range[2];
   const int lo = k * kForceChunk, hi = min(a.M, lo + kForceChunk);
-  const int b0 = a.mbody[lo], b1 = a.mbody[hi - 1];
-  for (int bd = b0; bd <= b1; ++bd) {
-    const BodyDev& B = a.bodies[bd];
-    const int l0 = max(lo, B.m0), l1 = min(hi, B.m1);
-    double fx = 0.0, fy = 0.0, tq = 0.0;
-    for (int l = l0 + (int)threadIdx.x; l < l1; l += NT) {
-      const double Fx = -a.ds[l] * (double)AN[2 * l], Fy = -a.ds[l] * (double)AN[2 * l + 1];
-      fx += Fx;
-      fy += Fy;
-      tq += (a.X[l] - B.xc[0]) * Fy - (a.Y[l] - B.xc[1]) * Fx;
-    }
-    block_sum3(fx, fy, tq, sh);
+  const int l = lo + (int)threadIdx.x;
+  int mb = -1;
+  double Fx = 0.0, Fy = 0.0, Tq = 0.0;
+  if (l < hi) {
+    const double d = -a.ds[l], X = a.X[l], Y = a.Y[l];
+    const double ax = (double)AN[2 * l], ay = (double)AN[2 * l + 1];
+    mb = a.mbody[l];
+    const BodyDev& B = a.bodies[mb];
+    Fx = d * ax;
+    Fy = d * ay;
+    Tq = (X - B.xc[0]) * Fy - (Y - B.xc[1]) * Fx;
+    if (l == lo) range[0] = mb;
+    if (l == hi - 1) range[1] = mb;
+  }
+  __syncthreads();
+  for (int bd = range[0]; bd <= range[1]; ++bd) {      // markers are stored body after body
+    double fx = mb == bd ? Fx : 0.0, fy = mb == bd ? Fy : 0.0, tq = mb == bd ? Tq : 0.0;
+    chunk_sum3(fx, fy, tq, sh);
     if (threadIdx.x == 0) {
       double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
       o[0] = fx; o[1] = fy; o[2] = tq;
     }
   }
+  __syncthreads();                                     // range is free for the next chunk
 }
 
 // Body totals: bodies rank, rank + nranks, .. by this CTA, fixed-shape
 // reduction over the chunks (which other CTAs may have written in this
 // launch: read past the L1 cache).
-template <int P, int NT>
+template <int P>
 __device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks, double* sh) {
   for (int bd = rank; bd < a.nb; bd += nranks) {
     BodyDev& B = a.bodies[bd];
     const int k0 = B.m0 / kForceChunk, k1 = (B.m1 - 1) / kForceChunk;
     double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-    for (int k = k0 + (int)threadIdx.x; k <= k1; k += NT) {
-      const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
-      f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
-    }
-    block_sum3(f0, f1, f2, sh);
+    if (threadIdx.x < kForceChunk)
+      for (int k = k0 + (int)threadIdx.x; k <= k1; k += kForceChunk) {
+        const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
+        f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
+      }
+    if (k0 != k1) chunk_sum3(f0, f1, f2, sh);          // one chunk: thread 0 has it
     if (threadIdx.x == 0) {
       B.F_ib[0] = f0;
       B.F_ib[1] = f1;
@@ -761,7 +780,7 @@ __device__ __forceinline__ void ib_phase_final(const IbArgs<P>& a, int tid, int 
       a.bq[8 * b + 7] = dy;
     }
   }
-  for (int k = rank; k < (M + kForceChunk - 1) / kForceChunk; k += nranks) ib_force_chunk<P, NT>(a, AN, k, sh);
+  for (int k = rank; k < (M + kForceChunk - 1) / kForceChunk; k += nranks) ib_force_chunk<P>(a, AN, k, sh);
 }
 
 // r^N is complete: a non-finite residual means the state has diverged; one
@@ -806,7 +825,7 @@ __device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, in
     }
   }
 
-  ib_force_total<P, NT>(a, rank, nranks, sh);
+  ib_force_total<P>(a, rank, nranks, sh);
 }
 
 // Folds the CTA's warp maxima in red[] into *dst (integer maximum of the
@@ -838,7 +857,7 @@ template <int P, int PAR, int NT>
 __device__ void ib_step_body(const IbArgs<P>& a, int rank, int nranks) {
   typedef typename Prec<P>::R R;
   __shared__ R red[NT / 32];
-  __shared__ double sh[96];
+  __shared__ double sh[kChunkSumShared];
   const int tid = rank * NT + threadIdx.x;
   const int nth = nranks * NT;
   const int rtid = nth - 1 - tid;                  // band work starts from the other end
