@@ -104,7 +104,8 @@ __device__ __forceinline__ void signal_done(unsigned int* ctr) {
 }
 
 // Collide+stream of rows [y0, y1) of one case: warps take the row spans in
-// turn; threads then take the extrapolation columns of those rows.
+// turn; threads then take the edge nodes (odd step) and the extrapolation
+// columns of those rows.
 template <int P, int PAR, bool MACRO, bool MRT>
 __device__ __noinline__ void batch_tile(const IbArgs<P>& a, int y0, int y1) {
   constexpr int VEC = PAR ? VecTraits<P>::VEC_ODD : VecTraits<P>::VEC;
@@ -114,6 +115,24 @@ __device__ __noinline__ void batch_tile(const IbArgs<P>& a, int y0, int y1) {
   const int lane = threadIdx.x & 31;
   for (int sp = threadIdx.x >> 5; sp < nspan; sp += kBatchThreads / 32)
     k1_span<P, PAR, MACRO, K1_ALL, MRT>(g, a.c, a.A, a.mac, nullptr, 0, y0 + sp / wpr, sp % wpr, lane);
+  if (PAR == 1) {
+    const OddEdge e = odd_edge<VEC>(g);
+    const int lo = e.wall_rows ? max(y0, 1) : y0, hi = e.wall_rows ? min(y1, g.ny - 1) : y1;
+    const int cols = max(hi - lo, 0) * e.ncol;
+    const int low = e.wall_rows && y0 == 0 ? g.nx : 0, high = e.wall_rows && y1 == g.ny ? g.nx : 0;
+    for (int q = threadIdx.x; q < cols + low + high; q += kBatchThreads) {
+      int x, y;
+      if (q < cols) {
+        y = lo + q / e.ncol;
+        x = q % e.ncol;
+        if (x >= e.left) x += e.right - e.left;
+      } else {
+        y = q < cols + low ? 0 : g.ny - 1;
+        x = q - cols - (q < cols + low ? 0 : low);
+      }
+      k1_edge_xy<P, MACRO, K1_ALL, MRT>(g, a.c, a.A, a.mac, nullptr, 0, x, y);
+    }
+  }
   if (has_nee(g)) {
     const int rows = y1 - y0;
     for (int q = threadIdx.x; q < 2 * rows; q += kBatchThreads)

@@ -248,4 +248,37 @@ __device__ __forceinline__ typename Prec<P>::R post_stream(
   return v;
 }
 
+// The nine post-stream populations of (x, y).  The locations are worked out
+// and the loads issued one after another without using a value in between,
+// so that the nine loads are in flight together.  (The slot that holds
+// f_i has the weight of direction i.)
+template <int P>
+__device__ __forceinline__ void post_stream9(const Geom& g, const StepConsts<typename Prec<P>::R>& c,
+                                             const typename Prec<P>::S* A, int parity, int x, int y,
+                                             typename Prec<P>::R (&p)[9]) {
+  typedef typename Prec<P>::R R;
+  typename Prec<P>::S v[9];
+  R wall[9];
+  unsigned int stored = 0;                  // bit i: f_i is read (else the inlet equilibrium)
+  const bool inlet = x == 0 && g.bc[0] == BC_INLET;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    v[i] = typename Prec<P>::S(0.0f);
+    wall[i] = R(0);
+    if (inlet) continue;
+    if (parity == 0) {
+      v[i] = A[slot_index(g, i, x, y)];
+      stored |= 1u << i;
+      continue;
+    }
+    int sx, sy, slot, ws;
+    if (!locE(g, x, y, i, sx, sy, slot, ws)) continue;
+    v[i] = A[slot_index(g, slot, sx, sy)];
+    stored |= 1u << i;
+    if (ws >= 0) wall[i] = c.wall[ws][i];
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) p[i] = (stored >> i & 1u) ? Prec<P>::ld(v[i], i) + wall[i] : c.feq_in[i];
+}
+
 }  // namespace ibm

@@ -173,9 +173,7 @@ __device__ void odd_boundary(const Geom& g, const StepConsts<typename Prec<P>::R
   for (int q = 0; q < nn; ++q) {
     const int xq = x + q;
     R p[9], rho, jx, jy;
-    long long where;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) p[i] = post_stream<P>(g, c, A, 1, xq, y, i, where);
+    post_stream9<P>(g, c, A, 1, xq, y, p);
     if (xq == 0 && g.bc[0] == BC_INLET) {
 #pragma unroll
       for (int i = 0; i < 9; ++i) ps[q][i] = c.feq_in[i];
@@ -297,6 +295,17 @@ __device__ __forceinline__ void collide_vec(const Geom& g, const StepConsts<type
   }
 }
 
+// d_i -> (d_i + w_i) - w_i, a branch of its own (never select instructions in
+// the spans that do not need it).
+template <int VEC, class R>
+__device__ __forceinline__ void full_round(R (&p)[9][VEC]) {
+  asm volatile("" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) p[i][k] = __fsub_rn(__fadd_rn((float)p[i][k], wgt<float>(i)), wgt<float>(i));
+}
+
 // Even step for the VEC nodes x0.. of row y (all inside the lattice):
 // aligned vector loads of A[i], vector stores to A[opp(i)].  A lane with
 // `skip` set (its nodes lie in a band segment, which another kernel streams)
@@ -338,11 +347,13 @@ __device__ __forceinline__ void even_vec(const Geom& g, const StepConsts<typenam
 // the neighbouring span or to a skipped lane are read or written with
 // scalar accesses by the thread whose node owns the slot (the lanes at the
 // ends of each run of active lanes), so no slot of another node is written.
+// full (16-bit storage, the same for the whole warp): round as the scalar
+// path does, which forms f_i = w_i + d_i on either side of the collision.
 template <int P, bool MACRO, bool MRT>
 __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename Prec<P>::R>& c,
                                         typename Prec<P>::S* __restrict__ A,
                                         typename Prec<P>::R* __restrict__ mac, int x0, int y, int lane,
-                                        bool skip) {
+                                        bool skip, bool full) {
   typedef typename Prec<P>::S S;
   typedef typename Prec<P>::R R;
   constexpr int VEC = VecTraits<P>::VEC_ODD;
@@ -383,7 +394,9 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
       p[i][VEC - 1] = Prec<P>::ldv(right, sl);
     }
   }
+  if (sizeof(S) == 2 && full) full_round<VEC>(p);
   collide_vec<P, MACRO, MRT, VEC>(g, c, p, mac, x0, y, !skip);
+  if (sizeof(S) == 2 && full) full_round<VEC>(p);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const int ty = cy(i) > 0 ? yp : (cy(i) < 0 ? ym : y);
@@ -430,16 +443,83 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
   }
 }
 
+// ------------------------------------------------------------------ edges
+// Nodes of the odd step that the vector path leaves out: every node of a row
+// on a closed y side; in the other rows the first vector of a closed x side
+// and the vectors from the last closed columns (two before an outlet) or the
+// row's ragged end on.  They are numbered, wall rows first, and go one per
+// thread through the boundary rules, in blocks (or thread strides) of their
+// own: beside the vector path they cost it registers, and whole spans of them,
+// four nodes in turn per lane, made the odd step of a 1600 x 800 FP32 channel
+// 46.5 us against 13.9 for the even one (now 22.2; a 1001 x 777 closed box in
+// FP16 storage 16.4 -> 8.2 us a step).
+struct OddEdge {
+  int wall_rows;       // 1: rows 0 and ny - 1 are closed
+  int left, right;     // vectors at x0 < left or x0 >= right are edge nodes
+  int ncol;            // edge nodes of any other row
+  int special;         // first node from the right that needs the boundary rules (nx: none)
+};
+template <int VEC>
+__host__ __device__ __forceinline__ OddEdge odd_edge(const Geom& g) {
+  OddEdge e;
+  const bool closed_x = g.bc[0] != BC_PERIODIC;
+  e.special = closed_x ? g.nx - ((g.bc[1] == BC_OUTLET || g.bc[1] == BC_OUTLET_NEE) ? 2 : 1) : g.nx;
+  e.wall_rows = g.bc[2] != BC_PERIODIC;
+  e.left = closed_x ? VEC : 0;
+  e.right = e.special / VEC * VEC;
+  if (e.right < e.left) e.right = e.left;
+  e.ncol = e.left + (g.nx > e.right ? g.nx - e.right : 0);
+  return e;
+}
+// Rows of column edge nodes, and edge nodes in all.
+__host__ __device__ __forceinline__ int edge_rows(const Geom& g, const OddEdge& e) {
+  return e.wall_rows ? g.ny - 2 : g.ny;
+}
+__host__ __device__ __forceinline__ long long edge_nodes(const Geom& g, const OddEdge& e) {
+  return (e.wall_rows ? 2LL * g.nx : 0LL) + (long long)edge_rows(g, e) * e.ncol;
+}
+
+template <int P, bool MACRO, int MODE, bool MRT>
+__device__ __forceinline__ void k1_edge_xy(const Geom& g, const StepConsts<typename Prec<P>::R>& c,
+                                           typename Prec<P>::S* __restrict__ A,
+                                           typename Prec<P>::R* __restrict__ mac, const int* __restrict__ segflag,
+                                           int nseg_x, int x, int y) {
+  if (x >= g.nx || nee_column(g, x)) return;                  // k_open_columns streams those
+  if (MODE == K1_MAIN && segflag[y * nseg_x + x / kSegW]) return;
+  odd_node<P, MACRO, MRT>(g, c, A, mac, x, y);
+}
+
+// Edge node number k of the lattice.
+template <int P, bool MACRO, int MODE, bool MRT>
+__device__ __forceinline__ void k1_edge_node(const Geom& g, const StepConsts<typename Prec<P>::R>& c,
+                                             typename Prec<P>::S* __restrict__ A,
+                                             typename Prec<P>::R* __restrict__ mac, const int* __restrict__ segflag,
+                                             int nseg_x, long long k) {
+  const OddEdge e = odd_edge<VecTraits<P>::VEC_ODD>(g);
+  const long long walls = e.wall_rows ? 2LL * g.nx : 0LL;
+  int x, y;
+  if (k < walls) {
+    y = k < g.nx ? 0 : g.ny - 1;
+    x = (int)(k < g.nx ? k : k - g.nx);
+  } else {
+    const int q = (int)(k - walls);
+    if (e.ncol == 0 || q / e.ncol >= edge_rows(g, e)) return;
+    y = q / e.ncol + (e.wall_rows ? 1 : 0);
+    x = q % e.ncol;
+    if (x >= e.left) x += e.right - e.left;
+  }
+  k1_edge_xy<P, MACRO, MODE, MRT>(g, c, A, mac, segflag, nseg_x, x, y);
+}
+
 // ------------------------------------------------------------------ spans
 // One warp's share of a collide+stream step: the span of 32 * VEC
 // consecutive nodes of row y that starts at node wrow * 32 * VEC (all 32
 // lanes of the warp call it together).  PAR 0: even step, 1: odd step.
 // MODE K1_ALL: every node.  MODE K1_MAIN: every node outside the 32-node
 // segments that hold band nodes (segflag).  Even step: per lane, aligned
-// vectors (ragged row ends node by node).  Odd step: spans without boundary
-// or ragged nodes take the vector path (lanes whose nodes lie in band
-// segments sit out); the others go node by node through the boundary-aware
-// path.  Extrapolation columns are left to open_column.
+// vectors (ragged row ends node by node).  Odd step: the vector path, with
+// the lanes sitting out whose nodes lie in band segments or are edge nodes
+// (k1_edge_node takes those).  Extrapolation columns are left to open_column.
 template <int P, int PAR, bool MACRO, int MODE, bool MRT>
 __device__ __forceinline__ void k1_span(const Geom& g, const StepConsts<typename Prec<P>::R>& c,
                                         typename Prec<P>::S* __restrict__ A,
@@ -463,23 +543,13 @@ __device__ __forceinline__ void k1_span(const Geom& g, const StepConsts<typename
     }
     return;
   }
-  const bool closed_x = g.bc[0] != BC_PERIODIC;
-  const int x_special =
-      closed_x ? ((g.bc[1] == BC_OUTLET || g.bc[1] == BC_OUTLET_NEE) ? g.nx - 2 : g.nx - 1) : g.nx;
-  const bool edge = (g.bc[2] != BC_PERIODIC && (y == 0 || y == g.ny - 1)) ||
-                    (closed_x && xw == 0) || (xw + 32 * VEC > x_special) || (xw + 32 * VEC > g.nx);
-  if (edge) {
-    for (int k = 0; k < VEC; ++k) {
-      const int x = x0 + k;
-      if (x >= g.nx) break;
-      if (MODE == K1_MAIN && segflag[y * nseg_x + x / kSegW]) continue;
-      if (nee_column(g, x)) continue;                          // k_open_columns
-      odd_node<P, MACRO, MRT>(g, c, A, mac, x, y);
-    }
-    return;
-  }
-  if (__all_sync(0xffffffffu, flagged)) return;               // the whole span is band segments
-  odd_vec<P, MACRO, MRT>(g, c, A, mac, x0, y, lane, flagged);
+  const OddEdge e = odd_edge<VEC>(g);
+  if (e.wall_rows && (y == 0 || y == g.ny - 1)) return;       // k1_edge_node's
+  const bool skip = flagged || x0 < e.left || x0 >= e.right;
+  if (__all_sync(0xffffffffu, skip)) return;                  // the whole span is band segments
+  // spans with edge nodes keep the scalar path's 16-bit rounding throughout
+  const bool full = (e.left > 0 && xw == 0) || xw + 32 * VEC > e.special;
+  odd_vec<P, MACRO, MRT>(g, c, A, mac, x0, y, lane, skip, full);
 }
 
 // ------------------------------------------------------------------ open sides
@@ -500,9 +570,7 @@ __device__ __forceinline__ void open_column(const Geom& g, const StepConsts<type
   if (g.bc[side] != (side == 0 ? BC_INLET_NEE : BC_OUTLET_NEE)) return;
   const int xb = side == 0 ? 0 : g.nx - 1, xf = side == 0 ? 1 : g.nx - 2;
   R pf[9], pb[9], ps[2][9];
-  long long where;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) pf[i] = post_stream<P>(g, c, A, PAR, xf, y, i, where);
+  post_stream9<P>(g, c, A, PAR, xf, y, pf);
   R rf, jxf, jyf;
   moments9<R>(pf, rf, jxf, jyf);
   const R inv = R(1) / rf;

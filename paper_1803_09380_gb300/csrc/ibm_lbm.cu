@@ -33,9 +33,8 @@ namespace ibm {
 //   (the correction-loop kernel streams those segments after correcting
 //   them).
 // Even step: per lane, aligned vectors (ragged row ends node by node).  Odd
-// step: spans without boundary or ragged nodes take the vector path (lanes
-// whose nodes lie in band segments sit out); the others go node by node
-// through the boundary-aware path.
+// step: the vector path; the first edge_rows rows of blocks take the edge
+// nodes instead, one per thread.
 // Threads per collide+stream block (whole warps per row span).  Two warps:
 // a correction-kernel CTA resident beside collide+stream then displaces
 // only the registers it needs, not whole 256-thread blocks (on the 4096^2
@@ -56,8 +55,19 @@ template <int P, int PAR, bool MACRO, int MODE, bool MRT>
 __global__ void __launch_bounds__(kK1Threads, k1_min_blocks(P, PAR)) k_collide_stream(Geom g, StepConsts<typename Prec<P>::R> c,
                                                         typename Prec<P>::S* __restrict__ A,
                                                         typename Prec<P>::R* __restrict__ mac,
-                                                        const int* __restrict__ segflag, int nseg_x) {
-  k1_span<P, PAR, MACRO, MODE, MRT>(g, c, A, mac, segflag, nseg_x, blockIdx.y,
+                                                        const int* __restrict__ segflag, int nseg_x,
+                                                        int edge_rows) {
+  int y = blockIdx.y;
+  if (PAR == 1) {
+    y -= edge_rows;
+    if (y < 0) {
+      k1_edge_node<P, MACRO, MODE, MRT>(
+          g, c, A, mac, segflag, nseg_x,
+          ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kK1Threads + threadIdx.x);
+      return;
+    }
+  }
+  k1_span<P, PAR, MACRO, MODE, MRT>(g, c, A, mac, segflag, nseg_x, y,
                                     (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31);
 }
 
@@ -174,13 +184,17 @@ static void launch_k1(const Ctx& h, const StepConsts<typename Prec<P>::R>& c, in
   constexpr int VEC = PAR ? VecTraits<P>::VEC_ODD : VecTraits<P>::VEC;
   const int warps_per_row = (h.geom.nx + 32 * VEC - 1) / (32 * VEC);
   constexpr int wpb = kK1Threads / 32;
-  const dim3 grid((warps_per_row + wpb - 1) / wpb, h.geom.ny);
-  if (mode == K1_MAIN) {
-    k_collide_stream<P, PAR, MACRO, K1_MAIN, MRT><<<grid, kK1Threads, 0, s>>>(
-        h.geom, c, A, mac, h.dsegflag, h.nseg_x);
-  } else {
-    k_collide_stream<P, PAR, MACRO, K1_ALL, MRT><<<grid, kK1Threads, 0, s>>>(
-        h.geom, c, A, mac, h.dsegflag, h.nseg_x);
+  const int bx = (warps_per_row + wpb - 1) / wpb;
+  const long long edge = PAR ? edge_nodes(h.geom, odd_edge<VEC>(h.geom)) : 0;
+  const long long per_row = (long long)bx * kK1Threads;
+  const int edge_rows = (int)((edge + per_row - 1) / per_row);
+  auto kern = mode == K1_MAIN ? k_collide_stream<P, PAR, MACRO, K1_MAIN, MRT>
+                              : k_collide_stream<P, PAR, MACRO, K1_ALL, MRT>;
+  if (edge_rows + h.geom.ny <= 65535) {
+    kern<<<dim3(bx, edge_rows + h.geom.ny), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, edge_rows);
+  } else {                                    // beyond the grid's limit: the edge nodes by themselves
+    kern<<<dim3(bx, edge_rows), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, edge_rows);
+    kern<<<dim3(bx, h.geom.ny), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, 0);
   }
 }
 
