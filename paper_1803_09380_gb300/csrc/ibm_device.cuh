@@ -134,38 +134,39 @@ __device__ __forceinline__ long long slot_index(const Geom& g, int k, int x, int
   return (long long)k * g.plane + (long long)y * g.nxp + x;
 }
 
+// The two maps below take a direction that is constant after unrolling and
+// use no branches, so nine directions cost a few hundred instructions.  (As
+// branchy loops over the sides they made kernels of up to 240 KB of code that
+// runs once per launch, and waiting for instructions was most of the time of
+// the boundary paths.)
+//
 // Where the post-stream population f_i(x, y) lives after an EVEN step.
-// Returns false for an inlet node (its state is the inlet equilibrium).
-// Otherwise (sx, sy, slot) is the stored location and wside >= 0 names a
-// bounce-back side whose wall term must be added when reading.
+// Returns false for an inlet node (its state is the inlet equilibrium) and
+// for a link from outside an open side.  Otherwise (sx, sy, slot) is the
+// stored location and wside >= 0 names a bounce-back side whose wall term
+// must be added when reading.
 __device__ __forceinline__ bool locE(const Geom& g, int x, int y, int i, int& sx, int& sy,
                                      int& slot, int& wside) {
-#pragma unroll 1
-  for (int depth = 0; depth < 2; ++depth) {
-    if (x == 0 && g.bc[0] == BC_INLET) return false;
-    int tx = x - cx(i), ty = y - cy(i);
-    int crx = -1, cry = -1;
-    if (tx < 0) { if (g.bc[0] == BC_PERIODIC) tx += g.nx; else crx = 0; }
-    else if (tx >= g.nx) { if (g.bc[1] == BC_PERIODIC) tx -= g.nx; else crx = 1; }
-    if (ty < 0) { if (g.bc[2] == BC_PERIODIC) ty += g.ny; else cry = 2; }
-    else if (ty >= g.ny) { if (g.bc[3] == BC_PERIODIC) ty -= g.ny; else cry = 3; }
-    wside = -1;
-    if (crx < 0 && cry < 0) { sx = tx; sy = ty; slot = opp(i); return true; }
-    bool open = (crx >= 0 && is_open(g.bc[crx])) || (cry >= 0 && is_open(g.bc[cry]));
-    if (open) {
-      if (crx == 1 && g.bc[1] == BC_OUTLET) { x = g.nx - 2; continue; }  // zero gradient
-      return false;
-    }
-    if (crx < 0 && g.bc[cry] == BC_FREESLIP) {       // specular off a y wall
-      sx = tx; sy = y; slot = opp(dir_of(cx(i), -cy(i))); return true;
-    }
-    if (cry < 0 && g.bc[crx] == BC_FREESLIP) {       // specular off an x wall
-      sx = x; sy = ty; slot = opp(dir_of(-cx(i), cy(i))); return true;
-    }
-    sx = x; sy = y; slot = i; wside = cry >= 0 ? cry : crx;   // bounce-back
-    return true;
-  }
-  return false;
+  const int ex = cx(i), ey = cy(i);
+  const int bx = g.bc[ex > 0 ? 0 : 1], by = g.bc[ey > 0 ? 2 : 3];
+  bool ox = ex != 0 && x == (ex > 0 ? 0 : g.nx - 1), oy = ey != 0 && y == (ey > 0 ? 0 : g.ny - 1);
+  const bool wx = ox && bx == BC_PERIODIC, wy = oy && by == BC_PERIODIC;
+  int tx = wx ? (ex > 0 ? g.nx - 1 : 0) : x - ex;
+  const int ty = wy ? (ey > 0 ? g.ny - 1 : 0) : y - ey;
+  // zero-gradient outlet: column nx - 2's population
+  const bool out = ex < 0 && ox && bx == BC_OUTLET;
+  const int xe = out ? g.nx - 2 : x;
+  if (out) tx = g.nx - 1;
+  ox = ox && !wx && !out;
+  oy = oy && !wy;
+  const bool fy = oy && !ox && by == BC_FREESLIP;       // specular off a y wall
+  const bool fx = ox && !oy && bx == BC_FREESLIP;       // specular off an x wall
+  const bool bb = (ox || oy) && !fx && !fy;             // bounce-back
+  sx = bb ? xe : (fx ? x : tx);
+  sy = bb || fy ? y : ty;
+  slot = bb ? i : (fy ? opp(dir_of(ex, -ey)) : (fx ? opp(dir_of(-ex, ey)) : opp(i)));
+  wside = bb ? (oy ? (ey > 0 ? 2 : 3) : (ex > 0 ? 0 : 1)) : -1;
+  return !(ox && is_open(bx)) && !(x == 0 && g.bc[0] == BC_INLET);
 }
 
 // Where the ODD step stores the post-collision f*_j(x, y): up to two
@@ -173,28 +174,26 @@ __device__ __forceinline__ bool locE(const Geom& g, int x, int y, int i, int& sx
 // the bounce-back side whose wall term is subtracted (or -1).
 struct OddTargets {
   int n;
-  int tx[2], ty[2], slot[2];
+  int tx, ty, slot;         // first target; the second is (nx - 1, ty, slot)
   int wside;
 };
 __device__ __forceinline__ OddTargets oddTargets(const Geom& g, int x, int y, int j) {
+  const int ex = cx(j), ey = cy(j);
+  const int bx = g.bc[ex > 0 ? 1 : 0], by = g.bc[ey > 0 ? 3 : 2];
+  bool ox = ex != 0 && x == (ex > 0 ? g.nx - 1 : 0), oy = ey != 0 && y == (ey > 0 ? g.ny - 1 : 0);
+  const bool wx = ox && bx == BC_PERIODIC, wy = oy && by == BC_PERIODIC;
+  const int tx = wx ? (ex > 0 ? 0 : g.nx - 1) : x + ex, ty = wy ? (ey > 0 ? 0 : g.ny - 1) : y + ey;
+  ox = ox && !wx;
+  oy = oy && !wy;
+  const bool fy = oy && !ox && by == BC_FREESLIP, fx = ox && !oy && bx == BC_FREESLIP;
+  const bool bb = (ox || oy) && !fx && !fy;
   OddTargets o;
-  o.n = 0; o.wside = -1;
-  int tx = x + cx(j), ty = y + cy(j);
-  int crx = -1, cry = -1;
-  if (tx < 0) { if (g.bc[0] == BC_PERIODIC) tx += g.nx; else crx = 0; }
-  else if (tx >= g.nx) { if (g.bc[1] == BC_PERIODIC) tx -= g.nx; else crx = 1; }
-  if (ty < 0) { if (g.bc[2] == BC_PERIODIC) ty += g.ny; else cry = 2; }
-  else if (ty >= g.ny) { if (g.bc[3] == BC_PERIODIC) ty -= g.ny; else cry = 3; }
-  int nx_ = 0, ny_ = 0, k = 0;
-  if (crx < 0 && cry < 0) { nx_ = tx; ny_ = ty; k = j; }
-  else if ((crx >= 0 && is_open(g.bc[crx])) || (cry >= 0 && is_open(g.bc[cry]))) { return o; }
-  else if (crx < 0 && g.bc[cry] == BC_FREESLIP) { nx_ = tx; ny_ = y; k = dir_of(cx(j), -cy(j)); }
-  else if (cry < 0 && g.bc[crx] == BC_FREESLIP) { nx_ = x; ny_ = ty; k = dir_of(-cx(j), cy(j)); }
-  else { nx_ = x; ny_ = y; k = opp(j); o.wside = cry >= 0 ? cry : crx; }
-  o.tx[0] = nx_; o.ty[0] = ny_; o.slot[0] = k; o.n = 1;
-  if (g.bc[1] == BC_OUTLET && nx_ == g.nx - 2 && cx(k) < 0) {
-    o.tx[1] = g.nx - 1; o.ty[1] = ny_; o.slot[1] = k; o.n = 2;
-  }
+  o.tx = bb || fx ? x : tx;
+  o.ty = bb || fy ? y : ty;
+  o.slot = bb ? opp(j) : (fy ? dir_of(ex, -ey) : (fx ? dir_of(-ex, ey) : j));
+  o.wside = bb ? (oy ? (ey > 0 ? 3 : 2) : (ex > 0 ? 1 : 0)) : -1;
+  const bool left = bb || fx ? ex > 0 : ex < 0;          // the stored population moves to -x
+  o.n = ox && is_open(bx) ? 0 : (g.bc[1] == BC_OUTLET && left && o.tx == g.nx - 2 ? 2 : 1);
   return o;
 }
 

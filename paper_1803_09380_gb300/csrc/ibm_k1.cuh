@@ -170,6 +170,7 @@ __device__ void odd_boundary(const Geom& g, const StepConsts<typename Prec<P>::R
   if (g.bc[1] == BC_OUTLET && x == g.nx - 1) return;   // done by the x = nx-2 thread
   const int nn = (g.bc[1] == BC_OUTLET && x == g.nx - 2) ? 2 : 1;
   R ps[2][9];
+#pragma unroll 1
   for (int q = 0; q < nn; ++q) {
     const int xq = x + q;
     R p[9], rho, jx, jy;
@@ -183,14 +184,16 @@ __device__ void odd_boundary(const Geom& g, const StepConsts<typename Prec<P>::R
     }
     if (MACRO) write_macro<R>(mac, (long long)g.nx * g.ny, (long long)y * g.nx + xq, rho, jx, jy);
   }
+#pragma unroll 1
   for (int q = 0; q < nn; ++q) {
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
-      OddTargets t = oddTargets(g, x + q, y, j);
+      const OddTargets t = oddTargets(g, x + q, y, j);
       R v = ps[q][j];
       if (t.wside >= 0) v -= c.wall[t.wside][j];
-      for (int k = 0; k < t.n; ++k)
-        A[slot_index(g, t.slot[k], t.tx[k], t.ty[k])] = Prec<P>::st(v, t.slot[k]);
+      const long long at = slot_index(g, t.slot, t.tx, t.ty);
+      if (t.n > 0) A[at] = Prec<P>::st(v, t.slot);
+      if (t.n > 1) A[at + 1] = Prec<P>::st(v, t.slot);         // tx = nx - 2: the outlet column beside it
     }
   }
 }
@@ -590,6 +593,7 @@ __device__ __forceinline__ void open_column(const Geom& g, const StepConsts<type
     collide_full<P, MRT>(pf, ps[1], rho, jx, jy, c);
     if (MACRO) write_macro<R>(mac, nn, (long long)y * g.nx + xf, rho, jx, jy);
   }
+#pragma unroll 1
   for (int q = 0; q < 2; ++q) {
     const int x = q == 0 ? xb : xf;
 #pragma unroll
@@ -597,10 +601,12 @@ __device__ __forceinline__ void open_column(const Geom& g, const StepConsts<type
       if (PAR == 0) {                                      // even step: node-local
         A[slot_index(g, opp(j), x, y)] = Prec<P>::st(ps[q][j], opp(j));
       } else {
-        OddTargets o = oddTargets(g, x, y, j);
+        const OddTargets o = oddTargets(g, x, y, j);
         R v = ps[q][j];
         if (o.wside >= 0) v -= c.wall[o.wside][j];
-        for (int k = 0; k < o.n; ++k) A[slot_index(g, o.slot[k], o.tx[k], o.ty[k])] = Prec<P>::st(v, o.slot[k]);
+        const long long at = slot_index(g, o.slot, o.tx, o.ty);
+        if (o.n > 0) A[at] = Prec<P>::st(v, o.slot);
+        if (o.n > 1) A[at + 1] = Prec<P>::st(v, o.slot);
       }
     }
   }
