@@ -289,7 +289,7 @@ void plan_slices(Ctx& c) {
   if (c.nm == 0 || c.any_moving || !c.band_collide || c.ib_phases != 0 || c.ib_threads != kIbThreads ||
       c.test_drop_arrival || c.desc.n_corr < 1 || c.desc.n_corr > slice_max_corr())
     return;
-  if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 4 * sizeof(int)))) return;
+  if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 8 * sizeof(int)))) return;
   const int asked = c.ib_grid_opt > 0 ? (c.nm + c.ib_grid - 1) / c.ib_grid : 0;
   for (int S = asked ? asked : slice_size(c); S >= 1; S /= 2) {
     const int count = (c.nm + S - 1) / S;
@@ -298,7 +298,7 @@ void plan_slices(Ctx& c) {
     c.sl_count = count;
     c.sl_mem = dev_alloc(c, slice_mem_bytes(c.prec, count));
     if (!c.sl_mem) break;
-    int stat[4] = {0, 0, 0, 0};
+    int stat[8] = {0};
     cudaError_t e = cudaMemsetAsync(c.dslstat, 0, sizeof(stat), c.stream);
     if (e == cudaSuccess) e = launch_slice_build(c, c.dslstat, c.stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(stat, c.dslstat, sizeof(stat), cudaMemcpyDeviceToHost, c.stream);
@@ -306,7 +306,10 @@ void plan_slices(Ctx& c) {
     if (e == cudaSuccess && stat[0] == 0) {
       c.sl_xmax = (stat[1] + 31) / 32 * 32;
       c.sl_x1max = (stat[2] + 31) / 32 * 32;
-      if (slice_smem(c.prec, c.desc.n_corr, c.sl_xmax, c.sl_x1max) > 0) {
+      c.sl_lmax = (stat[3] + 31) / 32 * 32;
+      c.sl_emax = stat[4];
+      c.sl_nseg = stat[5];
+      if (slice_smem(c) > 0) {
         c.sl_on = true;
         return;
       }

@@ -60,14 +60,19 @@ __device__ __forceinline__ int wrap_axis(int c, int n, bool periodic) {
 template <class R>
 __device__ __forceinline__ R nanmax(R a, R b) { return (a > b || a != a) ? a : b; }
 
+// Maxima of non-negative values (or NaN) through their bit patterns.
 template <class R> struct AtomicBits;
 template <> struct AtomicBits<float> {
-  static __device__ void max(float* a, float v) { atomicMax((unsigned int*)a, __float_as_uint(v)); }
+  typedef unsigned int U;
+  static __device__ void max_bits(U* a, float v) { atomicMax(a, __float_as_uint(v)); }
+  static __device__ void max(float* a, float v) { max_bits((U*)a, v); }
+  static __device__ float from_bits(U u) { return __uint_as_float(u); }
 };
 template <> struct AtomicBits<double> {
-  static __device__ void max(double* a, double v) {
-    atomicMax((unsigned long long*)a, (unsigned long long)__double_as_longlong(v));
-  }
+  typedef unsigned long long U;
+  static __device__ void max_bits(U* a, double v) { atomicMax(a, (U)__double_as_longlong(v)); }
+  static __device__ void max(double* a, double v) { max_bits((U*)a, v); }
+  static __device__ double from_bits(U u) { return __longlong_as_double((long long)u); }
 };
 // ------------------------------------------------------------------ band build
 // One item per (marker, stencil slot) or per band node.  The build runs in
@@ -557,23 +562,32 @@ template <int P>
 __device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typename Prec<P>::R* __restrict__ AN, int k,
                                                double* sh) {
   if (a.nb <= 0) return;
+  constexpr int kXc = 32;                              // body centres kept on hand
   __shared__ int range[2];
+  __shared__ double xc[2 * kXc];
   const int lo = k * kForceChunk, hi = min(a.M, lo + kForceChunk);
   const int l = lo + (int)threadIdx.x;
   int mb = -1;
-  double Fx = 0.0, Fy = 0.0, Tq = 0.0;
+  double Fx = 0.0, Fy = 0.0, Tq = 0.0, X = 0.0, Y = 0.0;
+  // one trip of loads: the centres do not wait for the markers' body numbers
+  if ((int)threadIdx.x < 2 * min(a.nb, kXc)) xc[threadIdx.x] = a.bodies[threadIdx.x >> 1].xc[threadIdx.x & 1];
   if (l < hi) {
-    const double d = -a.ds[l], X = a.X[l], Y = a.Y[l];
+    const double d = -a.ds[l];
     const double ax = (double)AN[2 * l], ay = (double)AN[2 * l + 1];
+    X = a.X[l];
+    Y = a.Y[l];
     mb = a.mbody[l];
-    const BodyDev& B = a.bodies[mb];
     Fx = d * ax;
     Fy = d * ay;
-    Tq = (X - B.xc[0]) * Fy - (Y - B.xc[1]) * Fx;
     if (l == lo) range[0] = mb;
     if (l == hi - 1) range[1] = mb;
   }
   __syncthreads();
+  if (mb >= 0) {
+    const double x0 = mb < kXc ? xc[2 * mb] : a.bodies[mb].xc[0], y0 = mb < kXc ? xc[2 * mb + 1] : a.bodies[mb].xc[1];
+    Tq = (X - x0) * Fy - (Y - y0) * Fx;
+  }
+#pragma unroll 1
   for (int bd = range[0]; bd <= range[1]; ++bd) {      // markers are stored body after body
     double fx = mb == bd ? Fx : 0.0, fy = mb == bd ? Fy : 0.0, tq = mb == bd ? Tq : 0.0;
     chunk_sum3(fx, fy, tq, sh);
@@ -585,22 +599,31 @@ __device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typenam
   __syncthreads();                                     // range is free for the next chunk
 }
 
-// Body totals: bodies rank, rank + nranks, .. by this CTA, fixed-shape
-// reduction over the chunks (which other CTAs may have written in this
-// launch: read past the L1 cache).
+// Body totals: a body per warp of this CTA and of the nranks that share the
+// work, fixed-shape reduction over the chunks (which other CTAs may have
+// written in this launch: read past the L1 cache).
 template <int P>
-__device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks, double* sh) {
-  for (int bd = rank; bd < a.nb; bd += nranks) {
+__device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks) {
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int bd = rank * nw + (threadIdx.x >> 5); bd < a.nb; bd += nranks * nw) {
     BodyDev& B = a.bodies[bd];
     const int k0 = B.m0 / kForceChunk, k1 = (B.m1 - 1) / kForceChunk;
     double f0 = 0.0, f1 = 0.0, f2 = 0.0;
-    if (threadIdx.x < kForceChunk)
-      for (int k = k0 + (int)threadIdx.x; k <= k1; k += kForceChunk) {
-        const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
-        f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
+#pragma unroll 1
+    for (int k = k0 + lane; k <= k1; k += 32) {
+      const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
+      f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
+    }
+    if (k0 != k1) {                                    // one chunk: lane 0 has it
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        f0 += __shfl_down_sync(0xffffffffu, f0, off);
+        f1 += __shfl_down_sync(0xffffffffu, f1, off);
+        f2 += __shfl_down_sync(0xffffffffu, f2, off);
       }
-    if (k0 != k1) chunk_sum3(f0, f1, f2, sh);          // one chunk: thread 0 has it
-    if (threadIdx.x == 0) {
+    }
+    if (lane == 0) {
       B.F_ib[0] = f0;
       B.F_ib[1] = f1;
       B.T_ib = f2;
@@ -825,7 +848,7 @@ __device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, in
     }
   }
 
-  ib_force_total<P>(a, rank, nranks, sh);
+  ib_force_total<P>(a, rank, nranks);
 }
 
 // Folds the CTA's warp maxima in red[] into *dst (integer maximum of the

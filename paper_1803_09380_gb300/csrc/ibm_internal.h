@@ -137,8 +137,10 @@ struct Ctx {
   bool sl_on = false;                        // steps run on the slices
   int sl_count = 0, sl_S = 0;                // slices, markers owned by each
   int sl_xmax = 0, sl_x1max = 0;             // largest local node counts
+  int sl_lmax = 0, sl_emax = 0;              // largest marker count and covering list
+  int sl_nseg = 0;                           // band segments (sizes the band grid)
   void* sl_mem = nullptr;                    // the slices' lists
-  int* dslstat = nullptr;                    // [4] build status
+  int* dslstat = nullptr;                    // [8] build status
   long long watch_due = 0;                   // steps since the last watchdog scan
 
   // CUDA graphs of one step, per parity and macro flag
@@ -331,10 +333,11 @@ void launch_body_update(const Ctx& h, cudaStream_t s);
 constexpr int kSliceMaxCount = 2048;
 size_t slice_mem_bytes(int prec, int count);
 // Builds the lists of h.sl_count slices of h.sl_S markers into h.sl_mem;
-// stat (device, 3 ints, zeroed): a slice did not fit, largest node counts.
+// stat (device, 8 ints, zeroed): a slice did not fit; largest node counts,
+// marker count and covering list; band segments.
 cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s);
 // Dynamic shared memory of the slice kernel (0: it does not fit).
-size_t slice_smem(int prec, int N, int xmax, int x1max);
+size_t slice_smem(const Ctx& h);
 int slice_max_corr();
 void launch_slice_loop(const Ctx& h, int parity, bool macro, cudaStream_t s);
 // Rigid motion of every moving body's markers to its current pose (Eqs. 41-42).

@@ -51,7 +51,9 @@ __device__ __forceinline__ int table_find(const int* keys, const unsigned short*
 // depth <= 1 markers, then the rest) and the local copies of weights, rows
 // and covering lists.  The order within a depth depends on the scheduling;
 // every sum runs in list order over marker ids, so results do not.
-// stat: [0] != 0 when a slice does not fit, [1], [2] largest node counts.
+// stat: [0] != 0 when a slice does not fit, [1], [2] largest node counts,
+// [3] largest marker count, [4] most markers that cover a node, [5] band
+// segments.
 template <class R>
 __global__ void __launch_bounds__(kSliceThreads) k_slice_build(SliceArgs<R> sl, int M, int N, const int* __restrict__ ctr,
                                                                const int* __restrict__ band_of,
@@ -69,6 +71,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_slice_build(SliceArgs<R> sl, 
   int* head = sl.head + (size_t)s * kSliceHead;
   for (int k = t; k < kSliceMarkHash; k += NT) mkey[k] = -1;
   for (int k = t; k < kSliceNodeHash; k += NT) nkey[k] = -1;
+  if (s == 0 && t == 0) stat[5] = ctr[CTR_NSEG];
   if (t == 0) { nm = 0; nn = 0; bad = ctr[CTR_ERR] & ~WARN_NOT_CONV; }   // a band that overflowed has no valid lists
   __syncthreads();
   const int m0 = s * sl.S, m1 = min(M, m0 + sl.S);
@@ -128,6 +131,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_slice_build(SliceArgs<R> sl, 
     if (nX1 > kSliceX1) bad = 1;
     atomicMax(&stat[1], nX);
     atomicMax(&stat[2], nX1);
+    atomicMax(&stat[3], nloc);
   }
   __syncthreads();
   if (bad) {
@@ -156,39 +160,52 @@ __global__ void __launch_bounds__(kSliceThreads) k_slice_build(SliceArgs<R> sl, 
           (unsigned short)(j < c ? table_find(mkey, mval, kSliceMarkHash, q.m) : k);
     }
   }
+  int most = 0;
   for (int k = t; k < nX1; k += NT) {
     const int b = sl.bid[(size_t)s * kSliceX1 + k];
     const int c = bcnt[b];
     if (c > kSliceEnt) atomicOr(&stat[0], 1);
+    most = max(most, c);
     sl.en[(size_t)s * kSliceX1 + k] = min(c, kSliceEnt);
-    for (int j = 0; j < min(c, kSliceEnt); ++j) {
-      const Ent<R> q = ent[(long long)b * kBandCap + j];
+    for (int j = 0; j < kSliceEnt; ++j) {                    // padded at weight zero
+      Ent<R> q;
+      q.w = R(0);
+      if (j < c) q = ent[(long long)b * kBandCap + j];
       sl.ew[((size_t)s * kSliceEnt + j) * kSliceX1 + k] = q.w;
       sl.ei[((size_t)s * kSliceEnt + j) * kSliceX1 + k] =
-          (unsigned short)table_find(mkey, mval, kSliceMarkHash, q.m);
+          (unsigned short)(j < c ? table_find(mkey, mval, kSliceMarkHash, q.m) : 0);
     }
   }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((t & 31) == 0) atomicMax(&stat[4], min(most, kSliceEnt));
 }
 
 // ------------------------------------------------------------------ correction
 // rho and j of U band nodes at once: their 9 U loads are in flight together.
+// Away from the sides (and in the even step everywhere) the locations are
+// constant offsets; false: some node needs the boundary rules instead.
+template <int P, int PAR>
+__device__ __forceinline__ bool plain_node(const Geom& g, int x, int y) {
+  return PAR == 0 || (x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1);
+}
 template <int P, int PAR, int U>
-__device__ __forceinline__ void gather_nodes(const IbArgs<P>& a, const int (&n)[U], typename Prec<P>::R (&rho)[U],
+__device__ __forceinline__ bool gather_nodes(const IbArgs<P>& a, const int (&n)[U], typename Prec<P>::R (&rho)[U],
                                              typename Prec<P>::R (&jx)[U], typename Prec<P>::R (&jy)[U]) {
   typedef typename Prec<P>::R R;
   typedef typename Prec<P>::S S;
   const Geom& g = a.g;
   S v[U][9];
-  bool plain[U];
+  bool all = true;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int y = n[u] / g.nx, x = n[u] - y * g.nx;
-    // away from the sides the locations are constant offsets
-    plain[u] = PAR == 0 || (x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1);
+    const bool plain = plain_node<P, PAR>(g, x, y);
+    all = all && plain;
     const long long base = (long long)y * g.nxp + x;
-    if (plain[u]) {
 #pragma unroll
-      for (int i = 0; i < 9; ++i)
+    for (int i = 0; i < 9; ++i) {
+      v[u][i] = S(0.0f);
+      if (plain)
         v[u][i] = PAR == 0 ? a.A[i * g.plane + base]
                            : a.A[opp(i) * g.plane + base - (long long)cy(i) * g.nxp - cx(i)];
     }
@@ -196,45 +213,114 @@ __device__ __forceinline__ void gather_nodes(const IbArgs<P>& a, const int (&n)[
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     R p[9];
-    if (plain[u]) {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) p[i] = Prec<P>::ld(v[u][i], PAR == 0 ? i : opp(i));
-    } else {
-      const int y = n[u] / g.nx, x = n[u] - y * g.nx;
-      long long where;
-#pragma unroll 1
-      for (int i = 0; i < 9; ++i) p[i] = post_stream<P>(g, a.c, a.A, PAR, x, y, i, where);
-    }
+    for (int i = 0; i < 9; ++i) p[i] = Prec<P>::ld(v[u][i], PAR == 0 ? i : opp(i));
     moments9<R>(p, rho[u], jx[u], jy[u]);
   }
+  return all;
 }
 
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int P, int PAR>
-__global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
+__global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
   typedef typename Prec<P>::R R;
   typedef typename Vec2<R>::T V;
   constexpr int NT = kSliceThreads;
-  constexpr int U = sizeof(R) == 8 ? 1 : 2;
+  constexpr bool F64 = sizeof(R) == 8;
+  constexpr int U = F64 ? 2 : 4;                             // nodes gathered at once per thread
+  constexpr int kLevels = 11;                                // iterates of the history read at once
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = a.N;
-  V* hist = reinterpret_cast<V*>(smem_raw);                  // [N + 1][kSliceMarkers] A^n
-  R* nr = reinterpret_cast<R*>(hist + (size_t)(N + 1) * kSliceMarkers);   // [xmax] rho, jx, jy
-  R* njx = nr + sl.xmax;
-  R* njy = njx + sl.xmax;
-  R* sxx = njy + sl.xmax;                                    // [x1max] sum_n j^n j^n
-  R* sxy = sxx + sl.x1max;
-  R* syy = sxy + sl.x1max;
-  R* cm = syy + sl.x1max;                                    // [3][kSliceMarkers] C
-  __shared__ R red[kSliceMaxCorr + 2][NT / 32];
+  const int N = a.N, LM = sl.lmax, XM = sl.xmax, X1M = sl.x1max, EM = sl.emax;
+  const int SM = (sl.S + 3) & ~3;
+  V* hist = reinterpret_cast<V*>(smem_raw);                  // [N + 1][LM] A^n
+  V* djs = hist + (size_t)(N + 1) * LM;                      // [N + 1][SM] dj^n of the owned markers
+  V* jn = djs + (size_t)(N + 1) * SM;                      // FP64: [N + 1][X1M] spread A^n
+  R* nr = reinterpret_cast<R*>(jn + (F64 ? (size_t)(N + 1) * X1M : 0));   // [XM] rho, jx, jy
+  R* njx = nr + XM;
+  R* njy = njx + XM;
+  R* sxx = njy + XM;                                         // [X1M] sum_n j^n j^n
+  R* sxy = sxx + X1M;
+  R* syy = sxy + X1M;
+  R* cm = syy + X1M;                                         // [3][LM] C
+  R* dv = cm + 3 * LM;                                       // [kStencil][LM] W_l(x) / rho(x)
+  R* rso = dv + kStencil * LM;                                                  // [SM] rho* of the owned markers
+  R* sew = rso + SM;                          // [EM][X1M] covering lists
+  int* sen = reinterpret_cast<int*>(sew + (size_t)EM * X1M);
+  unsigned short* sei = reinterpret_cast<unsigned short*>(sen + X1M);
+  unsigned short* dk = sei + (size_t)EM * X1M;               // [kStencil][LM] their nodes
+  __shared__ typename AtomicBits<R>::U rmax[kSliceMaxCorr + 2];   // residual maxima, as bits
   __shared__ int depth[kSliceMaxCorr + 2];                   // markers of depth <= h
-  const int s = blockIdx.x, t = threadIdx.x, warp = t >> 5;
+  const int s = blockIdx.x, t = threadIdx.x;
   const int* head = sl.head + (size_t)s * kSliceHead;
   const int nown = head[0], nX1 = head[1], nX = head[2];
   const int own = head[4], nloc = head[4 + N], d1 = head[5];
   const size_t sm = (size_t)s * kSliceMarkers;
-  for (int k = t; k <= N; k += NT) depth[k] = head[4 + k];
+#pragma unroll 1
+  for (int k = t; k <= N; k += NT) {
+    depth[k] = head[4 + k];
+    rmax[k] = 0;
+  }
 
-  // the marker's weights are on their way while the nodes are gathered
+  // the gather's loads first, then what later phases read: the covering
+  // lists to shared memory, the marker's weights and G row to registers
+  {
+    const int* nid = sl.nid + (size_t)s * kSliceNodes;
+    bool all = true;
+#pragma unroll 1
+    for (int k = t; k < nX; k += NT * U) {
+      int n[U];
+      R r[U], jx[U], jy[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) n[u] = nid[k + u * NT < nX ? k + u * NT : k];
+      all = gather_nodes<P, PAR, U>(a, n, r, jx, jy) && all;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k + u * NT < nX) {
+          nr[k + u * NT] = r[u];
+          njx[k + u * NT] = jx[u];
+          njy[k + u * NT] = jy[u];
+        }
+    }
+    if (!all) {                                              // this thread's nodes at the sides
+#pragma unroll 1
+      for (int k = t; k < nX; k += NT) {
+        const int n = nid[k], y = n / a.g.nx, x = n - y * a.g.nx;
+        if (plain_node<P, PAR>(a.g, x, y)) continue;
+        R p[9];
+        post_stream9<P>(a.g, a.c, a.A, PAR, x, y, p);
+        moments9<R>(p, nr[k], njx[k], njy[k]);
+      }
+    }
+  }
+  {
+    // a row of the lists per warp: EM of weights, EM of markers, the counts
+#pragma unroll 1
+    for (int j = t >> 5; j <= 2 * EM; j += NT / 32) {
+      const char* from;
+      char* to;
+      int bytes;
+      if (j < EM) {
+        from = (const char*)(sl.ew + ((size_t)s * kSliceEnt + j) * kSliceX1);
+        to = (char*)(sew + (size_t)j * X1M);
+        bytes = nX1 * (int)sizeof(R);
+      } else if (j < 2 * EM) {
+        from = (const char*)(sl.ei + ((size_t)s * kSliceEnt + j - EM) * kSliceX1);
+        to = (char*)(sei + (size_t)(j - EM) * X1M);
+        bytes = nX1 * (int)sizeof(short);
+      } else {
+        from = (const char*)(sl.en + (size_t)s * kSliceX1);
+        to = (char*)sen;
+        bytes = nX1 * (int)sizeof(int);
+      }
+#pragma unroll 1
+      for (int k = (t & 31) * 16; k < bytes; k += 512) copy16_async(to + k, from + k);
+    }
+  }
   R w[kStencil];
   unsigned int wi[kStencil / 2];
   R ux = R(0), uy = R(0);
@@ -247,29 +333,10 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
     ux = a.Ux[m];
     uy = a.Uy[m];
   }
-  {
-    const int* nid = sl.nid + (size_t)s * kSliceNodes;
-    for (int k = t; k < nX; k += NT * U) {
-      int n[U];
-      R r[U], jx[U], jy[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) n[u] = nid[k + u * NT < nX ? k + u * NT : k];
-      gather_nodes<P, PAR, U>(a, n, r, jx, jy);
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (k + u * NT < nX) {
-          nr[k + u * NT] = r[u];
-          njx[k + u * NT] = jx[u];
-          njy[k + u * NT] = jy[u];
-        }
-    }
-  }
-  // the marker's G row
   R rw[kRowHead];
   unsigned short ri[kRowHead];
   int rn = 0;
-  const int dj = N > 1 ? head[4 + N - 1] : 0;
-  const int drow = max(dj, own);                             // r^N needs the owned rows
+  const int drow = max(N > 1 ? head[4 + N - 1] : 0, own);    // r^N needs the owned rows
   if (t < drow) {
     rn = sl.rn[sm + t];
 #pragma unroll
@@ -282,7 +349,6 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
 
   // rho*, J*^0, b = A^1 (Eq. 22b, Eq. 28 in moment form)
   R rs = R(1), bx = R(0), by = R(0);
-  R rmax = R(0);
   if (t < nloc) {
     R jx = R(0), jy = R(0);
     rs = R(0);
@@ -292,6 +358,10 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
       rs += w[q] * nr[k];
       jx += w[q] * njx[k];
       jy += w[q] * njy[k];
+      if (t < d1) {
+        dv[q * LM + t] = w[q];
+        dk[q * LM + t] = (unsigned short)k;
+      }
     }
     bx = rs * ux - jx;
     by = rs * uy - jy;
@@ -300,93 +370,156 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
     b.x = bx;
     b.y = by;
     hist[t] = z;
-    hist[kSliceMarkers + t] = b;
-    if (t < own) rmax = (R)(sqrt(bx * bx + by * by) / rs);
+    hist[LM + t] = b;
+    if (t < own) {
+      djs[t] = b;
+      rso[t] = rs;
+    }
   }
-  if (warp * 32 < own) warp_max_to<R>(rmax, red[0]);
   __syncthreads();
 
-  // A^{n+1} = A^n + b - G A^n, to depth N - n; r^n of the owned markers
+  // A^{n+1} = A^n + b - G A^n, to depth N - n; dj^n of the owned markers (the
+  // last pass only forms dj^N)
   R ax = bx, ay = by;
-  auto row = [&](const V* An, R& djx, R& djy) {
-    R sx = R(0), sy = R(0);
-#pragma unroll
-    for (int j = 0; j < kRowHead; ++j) {
-      const V v = An[ri[j]];
-      sx += rw[j] * v.x;
-      sy += rw[j] * v.y;
-    }
-    for (int j = kRowHead; j < rn; ++j) {
-      const V v = An[sl.ri[((size_t)s * kSliceRow + j) * kSliceMarkers + t]];
-      const R wj = sl.rw[((size_t)s * kSliceRow + j) * kSliceMarkers + t];
-      sx += wj * v.x;
-      sy += wj * v.y;
-    }
-    djx = bx - sx;
-    djy = by - sy;
-  };
+#pragma unroll 1
   for (int n = 1; n <= N; ++n) {
-    const V* An = hist + (size_t)n * kSliceMarkers;
-    // the last pass only forms r^N
-    const int active = n < N ? depth[N - n] : own;
-    rmax = R(0);
-    if (t < active) {
-      R djx, djy;
-      row(An, djx, djy);
+    const V* An = hist + (size_t)n * LM;
+    if (t < (n < N ? depth[N - n] : own)) {
+      R sx = R(0), sy = R(0);
+#pragma unroll
+      for (int j = 0; j < kRowHead; ++j) {
+        const V v = An[ri[j]];
+        sx += rw[j] * v.x;
+        sy += rw[j] * v.y;
+      }
+#pragma unroll 1
+      for (int j = kRowHead; j < rn; ++j) {
+        const V v = An[sl.ri[((size_t)s * kSliceRow + j) * kSliceMarkers + t]];
+        const R wj = sl.rw[((size_t)s * kSliceRow + j) * kSliceMarkers + t];
+        sx += wj * v.x;
+        sy += wj * v.y;
+      }
+      V dj;
+      dj.x = bx - sx;
+      dj.y = by - sy;
+      if (t < own) djs[(size_t)n * SM + t] = dj;
       if (n < N) {
-        ax = ax + djx;
-        ay = ay + djy;
+        ax = ax + dj.x;
+        ay = ay + dj.y;
         V v;
         v.x = ax;
         v.y = ay;
-        hist[(size_t)(n + 1) * kSliceMarkers + t] = v;
+        hist[(size_t)(n + 1) * LM + t] = v;
       }
-      if (t < own) rmax = (R)(sqrt(djx * djx + djy * djy) / rs);
     }
-    if (warp * 32 < own) warp_max_to<R>(rmax, red[n]);
+    if (n == N) copy_async_wait();
     __syncthreads();
+  }
+
+  // r^n = max |dj^n| / rho* of the owned markers.  FP32: an n per warp; FP64:
+  // (n, marker) pairs fill the warps
+  if (F64) {
+#pragma unroll 1
+    for (int k = t; k < (N + 1) * own; k += NT) {
+      const int n = k / own, l = k - n * own;
+      const V d = djs[(size_t)n * SM + l];
+      AtomicBits<R>::max_bits(&rmax[n], nanmax(R(0), (R)(sqrt(d.x * d.x + d.y * d.y) / rso[l])));
+    }
+  } else {
+#pragma unroll 1
+    for (int n = t >> 5; n <= N; n += NT / 32) {
+      unsigned int m = 0;
+#pragma unroll 1
+      for (int l = t & 31; l < own; l += 32) {
+        const V d = djs[(size_t)n * SM + l];
+        m = max(m, __float_as_uint(nanmax(0.0f, (float)(sqrt(d.x * d.x + d.y * d.y) / rso[l]))));
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if ((t & 31) == 0) rmax[n] = m;
+    }
+  }
+  // W_l(x) / rho(x) of the depth <= 1 markers, spread over all threads
+#pragma unroll 1
+  for (int k = t; k < kStencil * d1; k += NT) {
+    const int at = k / d1 * LM + k % d1;
+    dv[at] = dv[at] / nr[dk[at]];
   }
 
   // per node of a depth <= 1 marker: sum_n j^n j^n; per owned node the summed
   // momentum correction D^N
-  for (int k = t; k < nX1; k += NT) {
-    const int cnt = sl.en[(size_t)s * kSliceX1 + k];
-    R ew[8];
-    unsigned short ei[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (j < cnt) {
-        ew[j] = sl.ew[((size_t)s * kSliceEnt + j) * kSliceX1 + k];
-        ei[j] = sl.ei[((size_t)s * kSliceEnt + j) * kSliceX1 + k];
+  if (F64) {
+    // (node, n) pairs fill the warps; the sums over n follow in order
+#pragma unroll 1
+    for (int k = t; k < (N + 1) * nX1; k += NT) {
+      const int n = k / nX1, x = k - n * nX1;
+      if (n == N && x >= nown) continue;
+      const int cnt = sen[x];
+      const V* An = hist + (size_t)n * LM;
+      V p;
+      p.x = p.y = R(0);
+#pragma unroll 1
+      for (int j = 0; j < cnt; ++j) {
+        const R wj = sew[(size_t)j * X1M + x];
+        const V v = An[sei[(size_t)j * X1M + x]];
+        p.x += wj * v.x;
+        p.y += wj * v.y;
       }
+      jn[(size_t)n * X1M + x] = p;
+    }
+    __syncthreads();
+  }
+#pragma unroll 1
+  for (int k = t; k < nX1; k += NT) {
     const R j0x = njx[k], j0y = njy[k];
     R axx = R(0), axy = R(0), ayy = R(0);
-    const int last = k < nown ? N : N - 1;
-    for (int n = 0; n <= last; ++n) {
-      const V* An = hist + (size_t)n * kSliceMarkers;
-      R px = R(0), py = R(0);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j < cnt) {
-          const V v = An[ei[j]];
-          px += ew[j] * v.x;
-          py += ew[j] * v.y;
-        }
-      for (int j = 8; j < cnt; ++j) {
-        const V v = An[sl.ei[((size_t)s * kSliceEnt + j) * kSliceX1 + k]];
-        const R wj = sl.ew[((size_t)s * kSliceEnt + j) * kSliceX1 + k];
-        px += wj * v.x;
-        py += wj * v.y;
-      }
-      if (n < N) {
-        const R jx = j0x + px, jy = j0y + py;
+    R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
+    if (F64) {
+#pragma unroll 1
+      for (int n = 0; n < N; ++n) {
+        const V p = jn[(size_t)n * X1M + k];
+        const R jx = j0x + p.x, jy = j0y + p.y;
         axx += jx * jx;
         axy += jx * jy;
         ayy += jy * jy;
-      } else {
-        R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
-        o[6] = px;
-        o[7] = py;
+      }
+      if (k < nown) {
+        const V p = jn[(size_t)N * X1M + k];
+        o[6] = p.x;
+        o[7] = p.y;
+      }
+    } else {
+      // kLevels iterates at a time: their loads are independent, and the list
+      // is walked once
+      const int cnt = sen[k];
+#pragma unroll 1
+      for (int n0 = 0; n0 <= N; n0 += kLevels) {
+        V p[kLevels];
+#pragma unroll
+        for (int u = 0; u < kLevels; ++u) p[u].x = p[u].y = R(0);
+#pragma unroll 1
+        for (int j = 0; j < cnt; ++j) {
+          const R wj = sew[(size_t)j * X1M + k];
+          const V* An = hist + (size_t)n0 * LM + sei[(size_t)j * X1M + k];
+#pragma unroll
+          for (int u = 0; u < kLevels; ++u)
+            if (n0 + u <= N) {
+              const V v = An[(size_t)u * LM];
+              p[u].x += wj * v.x;
+              p[u].y += wj * v.y;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kLevels; ++u) {
+          if (n0 + u < N) {
+            const R jx = j0x + p[u].x, jy = j0y + p[u].y;
+            axx += jx * jx;
+            axy += jx * jy;
+            ayy += jy * jy;
+          } else if (n0 + u == N && k < nown) {
+            o[6] = p[u].x;
+            o[7] = p[u].y;
+          }
+        }
       }
     }
     sxx[k] = axx;
@@ -398,35 +531,17 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
   // C_l = N rho* U U - sum_x W_l(x) / rho(x) sum_n j^n j^n
   if (t < d1) {
     R pxx = R(0), pxy = R(0), pyy = R(0);
-#pragma unroll
+#pragma unroll 4
     for (int q = 0; q < kStencil; ++q) {
-      const int k = (q & 1) ? (int)(wi[q / 2] >> 16) : (int)(wi[q / 2] & 0xffffu);
-      const R v = w[q] / nr[k];
+      const int k = dk[q * LM + t];
+      const R v = dv[q * LM + t];
       pxx += v * sxx[k];
       pxy += v * sxy[k];
       pyy += v * syy[k];
     }
     cm[t] = R(N) * rs * ux * ux - pxx;
-    cm[kSliceMarkers + t] = R(N) * rs * ux * uy - pxy;
-    cm[2 * kSliceMarkers + t] = R(N) * rs * uy * uy - pyy;
-  }
-  __syncthreads();
-
-  // Eq. 27 summed: the second-moment correction of the owned nodes
-  for (int k = t; k < nown; k += NT) {
-    const int cnt = sl.en[(size_t)s * kSliceX1 + k];
-    R pxx = R(0), pxy = R(0), pyy = R(0);
-    for (int j = 0; j < cnt; ++j) {
-      const int m = sl.ei[((size_t)s * kSliceEnt + j) * kSliceX1 + k];
-      const R wj = sl.ew[((size_t)s * kSliceEnt + j) * kSliceX1 + k];
-      pxx += wj * cm[m];
-      pxy += wj * cm[kSliceMarkers + m];
-      pyy += wj * cm[2 * kSliceMarkers + m];
-    }
-    R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
-    o[3] = pxx;
-    o[4] = pxy;
-    o[5] = pyy;
+    cm[LM + t] = R(N) * rs * ux * uy - pxy;
+    cm[2 * LM + t] = R(N) * rs * uy * uy - pyy;
   }
   // A^N of the owned markers (the forces), the slice's residuals
   if (t < own) {
@@ -435,10 +550,28 @@ __global__ void __launch_bounds__(kSliceThreads) k_ib_slice(IbArgs<P> a, SliceAr
     v.y = ay;
     reinterpret_cast<V*>(a.Ah)[(long long)N * a.M + sl.mid[sm + t]] = v;
   }
-  for (int n = t; n <= N; n += NT) {
-    R m = R(0);
-    for (int k = 0; k < (own + 31) / 32; ++k) m = nanmax(m, red[n][k]);
-    sl.rpart[(size_t)s * (kSliceMaxCorr + 2) + n] = m;
+#pragma unroll 1
+  for (int n = t; n <= N; n += NT)
+    sl.rpart[(size_t)s * (kSliceMaxCorr + 2) + n] = AtomicBits<R>::from_bits(rmax[n]);
+  __syncthreads();
+
+  // Eq. 27 summed: the second-moment correction of the owned nodes
+#pragma unroll 1
+  for (int k = t; k < nown; k += NT) {
+    const int cnt = sen[k];
+    R pxx = R(0), pxy = R(0), pyy = R(0);
+#pragma unroll 1
+    for (int j = 0; j < cnt; ++j) {
+      const int m = sei[(size_t)j * X1M + k];
+      const R wj = sew[(size_t)j * X1M + k];
+      pxx += wj * cm[m];
+      pxy += wj * cm[LM + m];
+      pyy += wj * cm[2 * LM + m];
+    }
+    R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
+    o[3] = pxx;
+    o[4] = pxy;
+    o[5] = pyy;
   }
 }
 
@@ -455,23 +588,20 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
   typedef typename Prec<P>::S S;
   const Geom& g = a.g;
   S* __restrict__ A = a.A;
-  const bool special = PAR == 0 ? (x == 0 && g.bc[0] == BC_INLET) : needs_boundary_path(g, x, y);
   const int b = a.node2band[y * g.nx + x];
-  if (special) {
+  if (PAR == 1 && needs_boundary_path(g, x, y)) {
     if (b >= 0) {
       const R* q = a.bq + 8 * (long long)b;
+#pragma unroll
       for (int i = 0; i < 9; ++i) {
-        long long where;
-        const R v = post_stream<P>(g, a.c, A, PAR, x, y, i, where);
-        (void)v;
-        if (where < 0) continue;
-        const int slot = (int)(where / g.plane);
+        int sx = x, sy = y, slot = i, ws;
+        if (!locE(g, x, y, i, sx, sy, slot, ws)) continue;
+        S* at = A + slot_index(g, slot, sx, sy);
         const R df = feq_i<R>(i, R(0), q[6], q[7], q[3], q[4], q[5]);
-        A[where] = Prec<P>::st(Prec<P>::ld(A[where], slot) + df, slot);
+        *at = Prec<P>::st(Prec<P>::ld(*at, slot) + df, slot);
       }
     }
-    if (PAR == 0) even_node<P, MACRO, MRT>(g, a.c, A, a.mac, x, y);
-    else odd_node<P, MACRO, MRT>(g, a.c, A, a.mac, x, y);
+    odd_boundary<P, MACRO, MRT>(g, a.c, A, a.mac, x, y);
     return;
   }
   const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
@@ -497,6 +627,11 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
     }
   }
   collide_full<P, MRT>(p, ps, rho, jx, jy, a.c);
+  if (PAR == 0 && x == 0 && g.bc[0] == BC_INLET) {             // as even_node
+#pragma unroll
+    for (int i = 0; i < 9; ++i) ps[i] = a.c.feq_in[i];
+    rho = a.c.rho0; jx = a.c.rho0 * a.c.inlet_u[0]; jy = a.c.rho0 * a.c.inlet_u[1];
+  }
   if (MACRO) write_macro<R>(a.mac, (long long)g.nx * g.ny, (long long)y * g.nx + x, rho, jx, jy);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
@@ -514,13 +649,15 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
 // chain in it: with one trip of loads per chunk, a halving tree for the FP64
 // sums and the residuals in a block of their own it takes 10.8 us instead of
 // 20.4 on a 300^2 lattice with 1029 markers (cold caches).
+constexpr int kFinishThreads = kForceChunk;
 template <int P, int PAR, bool MACRO, bool MRT>
-__global__ void __launch_bounds__(256) k_band_finish(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
+__global__ void __launch_bounds__(kFinishThreads) k_band_finish(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
   typedef typename Prec<P>::R R;
   const int nchunk = (a.M + kForceChunk - 1) / kForceChunk, nfin = nchunk + 1;
   if (blockIdx.x == 0) {
     const int lane = threadIdx.x & 31;
-    for (int n = threadIdx.x >> 5; n <= a.N; n += 8) {
+#pragma unroll 1
+    for (int n = threadIdx.x >> 5; n <= a.N; n += kFinishThreads / 32) {
       R m = R(0);
       for (int k = lane; k < sl.count; k += 32) m = nanmax(m, sl.rpart[(size_t)k * (kSliceMaxCorr + 2) + n]);
 #pragma unroll
@@ -546,14 +683,16 @@ __global__ void __launch_bounds__(256) k_band_finish(IbArgs<P> a, SliceArgs<type
       __syncthreads();
       if (!last) return;
     }
-    ib_force_total<P>(a, 0, 1, sh);
+    ib_force_total<P>(a, 0, 1);
     return;
   }
   const Geom& g = a.g;
   const int nseg = a.ctr[CTR_NSEG];
   const int lane = threadIdx.x & (kSegW - 1);
-  const int nw = ((gridDim.x - nfin) * blockDim.x) / kSegW;
-  for (int k = ((blockIdx.x - nfin) * blockDim.x + threadIdx.x) / kSegW; k < nseg; k += nw) {
+  // blocks first, then their warps: few segments spread over all SMs
+  const int nblk = gridDim.x - nfin;
+#pragma unroll 1
+  for (int k = (threadIdx.x >> 5) * nblk + blockIdx.x - nfin; k < nseg; k += nblk * (kFinishThreads / 32)) {
     const int seg = a.seglist[k];
     const int y = seg / a.nseg_x, x = (seg - y * a.nseg_x) * kSegW + lane;
     if (x >= g.nx || nee_column(g, x)) continue;          // k_open_columns streams those
@@ -569,6 +708,8 @@ static SliceArgs<R> slice_args(const Ctx& h) {
   s.S = h.sl_S;
   s.xmax = h.sl_xmax;
   s.x1max = h.sl_x1max;
+  s.lmax = h.sl_lmax;
+  s.emax = h.sl_emax;
   slice_bytes<R>(h.sl_count, (unsigned char*)h.sl_mem, &s);
   return s;
 }
@@ -595,11 +736,12 @@ cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s) {
   return h.r_bytes == 8 ? slice_build_t<double>(h, stat, s) : slice_build_t<float>(h, stat, s);
 }
 
-// Shared memory of the slice kernel for these local node counts, or 0 when
-// the device cannot give it.
+// Shared memory of the slice kernel for the planned slices, or 0 when the
+// device cannot give it.
 template <int P>
-static size_t slice_smem_t(int N, int xmax, int x1max) {
-  const size_t need = slice_smem_bytes<typename Prec<P>::R>(xmax, x1max, N);
+static size_t slice_smem_t(const Ctx& h) {
+  const size_t need = slice_smem_bytes<typename Prec<P>::R>(h.sl_xmax, h.sl_x1max, h.sl_lmax, h.sl_emax, h.sl_S,
+                                                            h.desc.n_corr);
   constexpr size_t kMax = 200 * 1024;
   if (need > kMax) return 0;
   if (cudaFuncSetAttribute(k_ib_slice<P, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax) != cudaSuccess ||
@@ -610,12 +752,12 @@ static size_t slice_smem_t(int N, int xmax, int x1max) {
   return need;
 }
 
-size_t slice_smem(int prec, int N, int xmax, int x1max) {
-  switch (prec) {
-    case PREC_FP64: return slice_smem_t<PREC_FP64>(N, xmax, x1max);
-    case PREC_FP32: return slice_smem_t<PREC_FP32>(N, xmax, x1max);
-    case PREC_FP16_DEV: return slice_smem_t<PREC_FP16_DEV>(N, xmax, x1max);
-    default: return slice_smem_t<PREC_BF16_DEV>(N, xmax, x1max);
+size_t slice_smem(const Ctx& h) {
+  switch (h.prec) {
+    case PREC_FP64: return slice_smem_t<PREC_FP64>(h);
+    case PREC_FP32: return slice_smem_t<PREC_FP32>(h);
+    case PREC_FP16_DEV: return slice_smem_t<PREC_FP16_DEV>(h);
+    default: return slice_smem_t<PREC_BF16_DEV>(h);
   }
 }
 
@@ -624,13 +766,12 @@ static void slice_loop_t(const Ctx& h, int parity, bool macro, cudaStream_t s) {
   typedef typename Prec<P>::R R;
   IbArgs<P> a = make_ib_args<P>(h);
   SliceArgs<R> sl = slice_args<R>(h);
-  const size_t smem = slice_smem_bytes<R>(sl.xmax, sl.x1max, a.N);
+  const size_t smem = slice_smem_bytes<R>(sl.xmax, sl.x1max, sl.lmax, sl.emax, sl.S, a.N);
   const dim3 grid(sl.count), block(kSliceThreads);
   if (parity == 0) launch_prio_smem(k_ib_slice<P, 0>, grid, block, smem, s, h.ib_prio, a, sl);
   else launch_prio_smem(k_ib_slice<P, 1>, grid, block, smem, s, h.ib_prio, a, sl);
   const int nchunk = (h.nm + kForceChunk - 1) / kForceChunk;
-  const int need = (h.segcap * kSegW + 255) / 256;
-  const dim3 g2(1 + nchunk + std::max(1, std::min(need, 8 * h.ib_grid_max))), b2(256);
+  const dim3 g2(1 + nchunk + std::max(1, std::min(h.sl_nseg, 16 * h.ib_grid_max))), b2(kFinishThreads);
   auto go = [&](auto kern) { launch_prio(kern, g2, b2, s, h.ib_prio, a, sl); };
   if (a.c.mrt) {
     if (parity == 0) { if (macro) go(k_band_finish<P, 0, true, true>); else go(k_band_finish<P, 0, false, true>); }

@@ -24,7 +24,13 @@
 // What bounds it: latency.  The persistent kernel paid thirteen grid
 // barriers, each followed by dependent loads from L2; here the only global
 // round trips are the slice's lists and the gather, and an iteration is ten
-// shared-memory loads and a block barrier.
+// shared-memory loads and a block barrier.  The covering lists come to
+// shared memory by asynchronous copies behind the iterations, and the
+// residuals (a square root and a division each) are formed after the last
+// iteration, for all iterations at once.  In FP64, whose arithmetic issues
+// at two lanes a clock on an SM, work is dealt out so that whole warps are
+// filled: (node, iteration) pairs in the second moments.  Loops are kept
+// rolled: code that runs once per launch costs more to fetch than to execute.
 #pragma once
 
 #include "ibm_ib.cuh"
@@ -47,6 +53,7 @@ template <class R>
 struct SliceArgs {
   int count, S;                // slices, owned markers of each
   int xmax, x1max;             // largest local node counts (shared-memory strides)
+  int lmax, emax;              // largest marker count; most markers that cover a node
   int* head;                   // [count][kSliceHead]: owned nodes, nodes of depth <= 1
                                // markers, nodes, 0; then markers of depth <= h, h = 0 ..
   int* mid;                    // [count][kSliceMarkers] marker ids, by depth
@@ -91,17 +98,22 @@ inline size_t slice_bytes(int count, unsigned char* base, SliceArgs<R>* s) {
   t.rpart = (R*)take(n * (kSliceMaxCorr + 2) * sizeof(R));
   if (s) {
     t.count = s->count; t.S = s->S; t.xmax = s->xmax; t.x1max = s->x1max;
+    t.lmax = s->lmax; t.emax = s->emax;
     *s = t;
   }
   return used;
 }
 
-// Dynamic shared memory of one slice CTA: rho, j of the local nodes, their
-// second moments, the A history and the C of the depth <= 1 markers.
+// Dynamic shared memory of one slice CTA, in the order of its pieces: the A
+// history, the owned markers' dj^n, (FP64) j^n of the depth <= 1 markers'
+// nodes; rho, j of the nodes; sum_n j^n j^n; C; W / rho; rho* of the owned
+// markers; the covering lists' weights, counts and markers; the nodes of W / rho.
 template <class R>
-__host__ __device__ constexpr size_t slice_smem_bytes(int xmax, int x1max, int N) {
-  return sizeof(R) * ((size_t)3 * xmax + (size_t)3 * x1max + (size_t)(N + 1) * 2 * kSliceMarkers +
-                      (size_t)3 * kSliceMarkers);
+__host__ __device__ constexpr size_t slice_smem_bytes(int xmax, int x1max, int lmax, int emax, int S, int N) {
+  return 2 * sizeof(R) * ((size_t)(N + 1) * (lmax + ((S + 3) & ~3)) + (sizeof(R) == 8 ? (size_t)(N + 1) * x1max : 0)) +
+         sizeof(R) * ((size_t)3 * xmax + (size_t)3 * x1max + (size_t)3 * lmax + ((S + 3) & ~3)) +
+         (size_t)emax * x1max * (sizeof(R) + sizeof(short)) + (size_t)x1max * sizeof(int) +
+         (size_t)kStencil * lmax * (sizeof(R) + sizeof(short));
 }
 
 }  // namespace ibm
