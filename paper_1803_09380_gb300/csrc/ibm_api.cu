@@ -116,7 +116,7 @@ void destroy_graphs(Ctx& h) {
     if (h.graph_block[p]) { cudaGraphExecDestroy(h.graph_block[p]); h.graph_block[p] = nullptr; }
 }
 
-void enqueue_step(Ctx& h, int parity, bool macro, bool timing);
+void enqueue_step(Ctx& h, int parity, bool macro, bool timing, bool fprev = false, bool fnow = true);
 
 // Capture `count` consecutive steps starting at `parity` into one graph.
 cudaError_t capture_steps(Ctx& c, int parity, int count, bool macro_last, cudaGraphExec_t* out) {
@@ -124,7 +124,7 @@ cudaError_t capture_steps(Ctx& c, int parity, int count, bool macro_last, cudaGr
   cudaError_t e = cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
   for (int j = 0; j < count; ++j)
-    enqueue_step(c, parity ^ (j & 1), macro_last && j == count - 1, false);
+    enqueue_step(c, parity ^ (j & 1), macro_last && j == count - 1, false, j > 0, j == count - 1);
   e = cudaStreamEndCapture(c.stream, &graph);
   if (e != cudaSuccess) return e;
   // per-node priorities: the correction chain keeps its high priority inside
@@ -175,18 +175,21 @@ ibm_status ensure_io(Ctx* h, size_t doubles) {
 }
 
 // The launch sequence of one time step.  Without markers: one collide+stream
-// launch.  With markers the step forks: the correction-loop kernel (which
+// launch.  On slices: the correction and one kernel for everything else (the
+// timed form brackets the band-free collide+stream and keeps it apart).
+// Otherwise, with markers, the step forks: the correction-loop kernel (which
 // ends with collide+stream of the band row segments) runs on the
 // high-priority stream while collide+stream covers every band-free row
 // segment on the main stream; after the join, moving bodies are advanced
 // and re-binned.
-void enqueue_step(Ctx& h, int parity, bool macro, bool timing) {
+void enqueue_step(Ctx& h, int parity, bool macro, bool timing, bool fprev, bool fnow) {
   const bool t = timing && h.ev_used < kEventPairs;
   cudaEvent_t* e = t ? &h.ev[kEventsPerStep * h.ev_used] : nullptr;
   if (h.nm == 0) {
     if (t) cudaEventRecord(e[0], h.stream);
     launch_collide_stream(h, parity, macro, K1_ALL, h.stream);
     if (t) cudaEventRecord(e[1], h.stream);
+  } else if (!timing && launch_slice_step(h, parity, macro, fprev, fnow, h.stream)) {
   } else {
     cudaEventRecord(h.ev_fork, h.stream);
     cudaStreamWaitEvent(h.ib_stream, h.ev_fork, 0);
@@ -366,14 +369,14 @@ ibm_status upload_markers(Ctx* h) {
   IBM_ALLOC(h, c.dbnode, int*, c.bcap);
   IBM_ALLOC(h, c.dbcnt, int*, c.bcap);
   c.dent = dev_alloc(c, (R == 8 ? sizeof(Ent<double>) : sizeof(Ent<float>)) * (size_t)c.bcap * kBandCap);
-  IBM_ALLOC(h, c.dfpart, double*, (size_t)((M + kForceChunk - 1) / kForceChunk) * c.nb * 3);
+  IBM_ALLOC(h, c.dfpart, double*, (size_t)((M + kForceChunk - 1) / kForceChunk) * c.nb * 3 * 2);
   // correction-kernel CTAs: one for small boundaries (its grid barrier is a
   // block barrier, so such kernels of several lattices may run side by
   // side), one per SM otherwise
   choose_ib_grid(c);
   c.dbq = dev_alloc(c, R * 8 * (size_t)c.bcap);
   c.dmq = dev_alloc(c, R * 4 * (size_t)M);
-  c.dAh = dev_alloc(c, R * 2 * (size_t)M * (c.desc.n_corr + 1));
+  c.dAh = dev_alloc(c, R * 2 * (size_t)M * (c.desc.n_corr + 2));
   c.dCm = dev_alloc(c, R * 3 * (size_t)M);
   c.dG = dev_alloc(c, (R == 8 ? sizeof(Ent<double>) : sizeof(Ent<float>)) * (size_t)M * kGCap);
   IBM_ALLOC(h, c.dgcnt, int*, M);
@@ -400,7 +403,7 @@ ibm_status upload_markers(Ctx* h) {
   IBM_CK(h, cudaMemcpyAsync(c.dUy, uy.data(), R * M, cudaMemcpyHostToDevice, c.stream));
   IBM_CK(h, cudaMemcpyAsync(c.dbodies, c.hbodies.data(), sizeof(BodyDev) * c.nb,
                             cudaMemcpyHostToDevice, c.stream));
-  IBM_CK(h, cudaMemsetAsync(c.dAh, 0, R * 2 * (size_t)M * (c.desc.n_corr + 1), c.stream));
+  IBM_CK(h, cudaMemsetAsync(c.dAh, 0, R * 2 * (size_t)M * (c.desc.n_corr + 2), c.stream));
   IBM_CK(h, cudaMemsetAsync(c.dCm, 0, R * 3 * (size_t)M, c.stream));
   IBM_CK(h, cudaMemsetAsync(c.dG, 0, (R == 8 ? sizeof(Ent<double>) : sizeof(Ent<float>)) * (size_t)M * kGCap,
                             c.stream));
@@ -806,7 +809,7 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
         IBM_CK(h, cudaGetLastError());
       }
       c.parity ^= 1;
-      c.launches += kernels_per_step(c);
+      c.launches += kernels_per_step(c, timing);
       c.steps += 1;
       c.watch_due += 1;
       watchdog_if_due(c);

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kIbThreads) k_ib_jacobi(IbArgs<P> a, int n) {
 template <int P>
 __global__ void __launch_bounds__(kIbThreads) k_ib_final(IbArgs<P> a) {
   __shared__ typename Prec<P>::R red[kIbThreads / 32];
-  __shared__ double sh[kChunkSumShared];
+  __shared__ ForceShared<kIbThreads> sh;
   const int tid = blockIdx.x * kIbThreads + threadIdx.x, nth = gridDim.x * kIbThreads;
   ib_phase_final<P, kIbThreads>(a, tid, nth, nth - 1 - tid, min(a.ctr[CTR_NBAND], a.bcap), blockIdx.x,
                                 gridDim.x, red, sh);
@@ -114,10 +114,9 @@ __global__ void __launch_bounds__(kIbThreads) k_ib_final(IbArgs<P> a) {
 
 template <int P>
 __global__ void __launch_bounds__(kIbThreads) k_ib_moments(IbArgs<P> a) {
-  __shared__ double sh[kChunkSumShared];
-  if (blockIdx.x == 0 && threadIdx.x == 0) ib_check_resid<P>(a);
+  if (blockIdx.x == 0 && threadIdx.x == 0) ib_check_resid<P>(a, a.resid[a.N]);
   ib_phase_moments<P, kIbThreads>(a, blockIdx.x * kIbThreads + threadIdx.x, gridDim.x * kIbThreads,
-                                  blockIdx.x, gridDim.x, sh);
+                                  blockIdx.x, gridDim.x);
 }
 
 // The correction loop with its Jacobi iterations in one thread-block
@@ -145,13 +144,13 @@ template <int P, int NT>
 __global__ void __launch_bounds__(NT, 3) k_ib_post(IbArgs<P> a) {
   typedef typename Prec<P>::R R;
   __shared__ R red[NT / 32];
-  __shared__ double sh[kChunkSumShared];
+  __shared__ ForceShared<NT> sh;
   const int tid = blockIdx.x * NT + threadIdx.x, nth = gridDim.x * NT;
   ib_phase_final<P, NT>(a, tid, nth, nth - 1 - tid, min(a.ctr[CTR_NBAND], a.bcap), blockIdx.x, gridDim.x,
                         red, sh);
   grid_barrier<R>(a.bar, a.ctr, red, a.resid + a.N, a.cluster, a.bar_limit_ns, gridDim.x);
-  if (blockIdx.x == 0 && threadIdx.x == 0) ib_check_resid<P>(a);
-  ib_phase_moments<P, NT>(a, tid, nth, blockIdx.x, gridDim.x, sh);
+  if (blockIdx.x == 0 && threadIdx.x == 0) ib_check_resid<P>(a, a.resid[a.N]);
+  ib_phase_moments<P, NT>(a, tid, nth, blockIdx.x, gridDim.x);
 }
 
 __device__ __forceinline__ unsigned int cluster_rank() {

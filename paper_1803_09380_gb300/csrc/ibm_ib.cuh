@@ -256,7 +256,8 @@ struct IbArgs {
   const Ent<R>* G;
   const int* gcnt;
   R* mq;                      // [M][4]: rho*, b_x, b_y, pad
-  R* Ah;                      // [N+1][M][2] accumulated momentum deviations
+  R* Ah;                      // [N+2][M][2] accumulated momentum deviations (slices: A^N by step
+                              // parity in the last two levels)
   R* Cm;                      // [M][3]
   const R* Ux;
   const R* Uy;
@@ -267,7 +268,7 @@ struct IbArgs {
   const double* X;
   const double* Y;
   const double* ds;
-  double* fpart;              // [chunks][nb][3]
+  double* fpart;              // [2][chunks][nb][3] (the slices alternate by step parity)
   unsigned long long* bar;    // grid-barrier arrivals (monotonic)
   const int* node2band;       // [ny][nx] band index of a node, -1 outside the band
   int apply;                  // 1: apply the correction here; 0: k_band_collide applies it
@@ -466,13 +467,16 @@ __device__ __forceinline__ void warp_max_to(R v, R* red) {
 // thread 0; the tree's shape does not depend on the CTA's size.  FP64 adds
 // issue at two lanes a clock on an SM, so the halving tree (24 warp-wide
 // adds) is taken instead of a butterfly in every warp (60 and more).
+template <bool HALVED = false>                       // HALVED: thread t holds values t and t + 64 added
 __device__ __forceinline__ void chunk_sum3(double& a, double& b, double& c, double* sh) {
   static_assert(kForceChunk == 128, "the tree below adds 128 values");
   const int t = threadIdx.x;
-  if (t >= 64 && t < 128) { sh[t - 64] = a; sh[t] = b; sh[64 + t] = c; }
-  __syncthreads();
-  if (t < 64) { a += sh[t]; b += sh[64 + t]; c += sh[128 + t]; }
-  __syncthreads();
+  if (!HALVED) {
+    if (t >= 64 && t < 128) { sh[t - 64] = a; sh[t] = b; sh[64 + t] = c; }
+    __syncthreads();
+    if (t < 64) { a += sh[t]; b += sh[64 + t]; c += sh[128 + t]; }
+    __syncthreads();
+  }
   if (t >= 32 && t < 64) { sh[t - 32] = a; sh[t] = b; sh[32 + t] = c; }
   __syncthreads();
   if (t < 32) {
@@ -486,7 +490,14 @@ __device__ __forceinline__ void chunk_sum3(double& a, double& b, double& c, doub
   }
   __syncthreads();
 }
-constexpr int kChunkSumShared = 192;                 // doubles of shared memory it uses
+// Shared memory of the force sums in a CTA of NT threads.
+constexpr int kForceXc = 16;                         // body centres kept on hand
+template <int NT>
+struct ForceShared {
+  double sum[NT < kForceChunk ? 96 : 192];
+  double xc[2 * kForceXc];
+  int range[2], last;
+};
 
 template <class R> struct Vec2;
 template <> struct Vec2<float> { typedef float2 T; };
@@ -554,46 +565,71 @@ __device__ __forceinline__ void deviation(const Args& a, int l, const R* __restr
   djx = a.mq[4 * l + 1] - sx;
   djy = a.mq[4 * l + 2] - sy;
 }
+// Waits until the kernel that this one was launched behind (programmatic
+// dependent launch) has finished and its writes are visible; at once when the
+// launch had no such dependency.
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the kernel launched behind this one start.
+__device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Eq. 29: partial force and torque of each body over one fixed chunk of
-// kForceChunk markers (one CTA, a marker per thread), F_l = -ds_l A^N_l,
+// kForceChunk markers (one CTA of NT threads), F_l = -ds_l A^N_l,
 // T_l = (X_l - x_c) x F_l, FP64; the chunking does not depend on the grid, so
-// neither do the sums.
-template <int P>
+// neither do the sums.  WAIT: A^N comes from the kernel launched before.
+template <int P, int NT, bool WAIT>
 __device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typename Prec<P>::R* __restrict__ AN, int k,
-                                               double* sh) {
+                                               double* __restrict__ fpart, ForceShared<NT>& sh) {
   if (a.nb <= 0) return;
-  constexpr int kXc = 32;                              // body centres kept on hand
-  __shared__ int range[2];
-  __shared__ double xc[2 * kXc];
+  constexpr int kXc = kForceXc;
+  constexpr int H = NT < kForceChunk ? kForceChunk / NT : 1;   // markers per thread
+  static_assert(H <= 2, "at least half a chunk of threads");
+  int* range = sh.range;
+  double* xc = sh.xc;
   const int lo = k * kForceChunk, hi = min(a.M, lo + kForceChunk);
-  const int l = lo + (int)threadIdx.x;
-  int mb = -1;
-  double Fx = 0.0, Fy = 0.0, Tq = 0.0, X = 0.0, Y = 0.0;
+  int mb[H];
+  double F[H][3], X[H], Y[H], d[H];
   // one trip of loads: the centres do not wait for the markers' body numbers
   if ((int)threadIdx.x < 2 * min(a.nb, kXc)) xc[threadIdx.x] = a.bodies[threadIdx.x >> 1].xc[threadIdx.x & 1];
-  if (l < hi) {
-    const double d = -a.ds[l];
-    const double ax = (double)AN[2 * l], ay = (double)AN[2 * l + 1];
-    X = a.X[l];
-    Y = a.Y[l];
-    mb = a.mbody[l];
-    Fx = d * ax;
-    Fy = d * ay;
-    if (l == lo) range[0] = mb;
-    if (l == hi - 1) range[1] = mb;
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int l = lo + (int)threadIdx.x + h * NT;
+    mb[h] = -1;
+    d[h] = X[h] = Y[h] = 0.0;
+    if (l < hi) {
+      d[h] = -a.ds[l];
+      X[h] = a.X[l];
+      Y[h] = a.Y[l];
+      mb[h] = a.mbody[l];
+      if (l == lo) range[0] = mb[h];
+      if (l == hi - 1) range[1] = mb[h];
+    }
   }
+  if (WAIT) dependency_wait();
   __syncthreads();
-  if (mb >= 0) {
-    const double x0 = mb < kXc ? xc[2 * mb] : a.bodies[mb].xc[0], y0 = mb < kXc ? xc[2 * mb + 1] : a.bodies[mb].xc[1];
-    Tq = (X - x0) * Fy - (Y - y0) * Fx;
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int l = lo + (int)threadIdx.x + h * NT;
+    F[h][0] = F[h][1] = F[h][2] = 0.0;
+    if (mb[h] >= 0) {
+      const double x0 = mb[h] < kXc ? xc[2 * mb[h]] : a.bodies[mb[h]].xc[0];
+      const double y0 = mb[h] < kXc ? xc[2 * mb[h] + 1] : a.bodies[mb[h]].xc[1];
+      F[h][0] = d[h] * (double)AN[2 * l];
+      F[h][1] = d[h] * (double)AN[2 * l + 1];
+      F[h][2] = (X[h] - x0) * F[h][1] - (Y[h] - y0) * F[h][0];
+    }
   }
 #pragma unroll 1
   for (int bd = range[0]; bd <= range[1]; ++bd) {      // markers are stored body after body
-    double fx = mb == bd ? Fx : 0.0, fy = mb == bd ? Fy : 0.0, tq = mb == bd ? Tq : 0.0;
-    chunk_sum3(fx, fy, tq, sh);
+    double f[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      f[q] = mb[0] == bd ? F[0][q] : 0.0;
+      if (H == 2) f[q] += mb[H - 1] == bd ? F[H - 1][q] : 0.0;
+    }
+    chunk_sum3<H == 2>(f[0], f[1], f[2], sh.sum);
     if (threadIdx.x == 0) {
-      double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
-      o[0] = fx; o[1] = fy; o[2] = tq;
+      double* o = fpart + ((long long)k * a.nb + bd) * 3;
+      o[0] = f[0]; o[1] = f[1]; o[2] = f[2];
     }
   }
   __syncthreads();                                     // range is free for the next chunk
@@ -603,7 +639,8 @@ __device__ __forceinline__ void ib_force_chunk(const IbArgs<P>& a, const typenam
 // work, fixed-shape reduction over the chunks (which other CTAs may have
 // written in this launch: read past the L1 cache).
 template <int P>
-__device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks) {
+__device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int nranks, const double* fpart,
+                                               bool store = true) {
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int bd = rank * nw + (threadIdx.x >> 5); bd < a.nb; bd += nranks * nw) {
@@ -612,7 +649,7 @@ __device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int
     double f0 = 0.0, f1 = 0.0, f2 = 0.0;
 #pragma unroll 1
     for (int k = k0 + lane; k <= k1; k += 32) {
-      const double* o = a.fpart + ((long long)k * a.nb + bd) * 3;
+      const double* o = fpart + ((long long)k * a.nb + bd) * 3;
       f0 += __ldcg(o); f1 += __ldcg(o + 1); f2 += __ldcg(o + 2);
     }
     if (k0 != k1) {                                    // one chunk: lane 0 has it
@@ -623,7 +660,7 @@ __device__ __forceinline__ void ib_force_total(const IbArgs<P>& a, int rank, int
         f2 += __shfl_down_sync(0xffffffffu, f2, off);
       }
     }
-    if (lane == 0) {
+    if (lane == 0 && store) {
       B.F_ib[0] = f0;
       B.F_ib[1] = f1;
       B.T_ib = f2;
@@ -728,7 +765,7 @@ __device__ __forceinline__ void ib_phase_jacobi(const IbArgs<P>& a, int n, int t
 
 template <int P, int NT>
 __device__ __forceinline__ void ib_phase_final(const IbArgs<P>& a, int tid, int nth, int rtid, int nband, int rank,
-                                               int nranks, typename Prec<P>::R* red, double* sh) {
+                                               int nranks, typename Prec<P>::R* red, ForceShared<NT>& sh) {
   typedef typename Prec<P>::R R;
   const int M = a.M, N = a.N;
   // final phase: residual r^N; per band node the final spread D^N and
@@ -803,22 +840,21 @@ __device__ __forceinline__ void ib_phase_final(const IbArgs<P>& a, int tid, int 
       a.bq[8 * b + 7] = dy;
     }
   }
-  for (int k = rank; k < (M + kForceChunk - 1) / kForceChunk; k += nranks) ib_force_chunk<P>(a, AN, k, sh);
+  for (int k = rank; k < (M + kForceChunk - 1) / kForceChunk; k += nranks)
+    ib_force_chunk<P, NT, false>(a, AN, k, a.fpart, sh);
 }
 
 // r^N is complete: a non-finite residual means the state has diverged; one
 // above corr_tol is reported as a warning (one thread).
 template <int P>
-__device__ __forceinline__ void ib_check_resid(const IbArgs<P>& a) {
+__device__ __forceinline__ void ib_check_resid(const IbArgs<P>& a, typename Prec<P>::R rN) {
   typedef typename Prec<P>::R R;
-  const R rN = a.resid[a.N];
   if (!isfinite(rN)) atomicOr(&a.ctr[CTR_ERR], ERR_DIVERGED);
   else if (a.corr_tol > R(0) && rN > a.corr_tol) atomicOr(&a.ctr[CTR_ERR], WARN_NOT_CONV);
 }
 
 template <int P, int NT>
-__device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, int nth, int rank, int nranks,
-                                                 double* sh) {
+__device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, int nth, int rank, int nranks) {
   typedef typename Prec<P>::R R;
   const int M = a.M, N = a.N;
   // second-moment deviations summed over the iterations:
@@ -848,7 +884,7 @@ __device__ __forceinline__ void ib_phase_moments(const IbArgs<P>& a, int tid, in
     }
   }
 
-  ib_force_total<P>(a, rank, nranks);
+  ib_force_total<P>(a, rank, nranks, a.fpart);
 }
 
 // Folds the CTA's warp maxima in red[] into *dst (integer maximum of the
@@ -880,7 +916,7 @@ template <int P, int PAR, int NT>
 __device__ void ib_step_body(const IbArgs<P>& a, int rank, int nranks) {
   typedef typename Prec<P>::R R;
   __shared__ R red[NT / 32];
-  __shared__ double sh[kChunkSumShared];
+  __shared__ ForceShared<NT> sh;
   const int tid = rank * NT + threadIdx.x;
   const int nth = nranks * NT;
   const int rtid = nth - 1 - tid;                  // band work starts from the other end
@@ -901,8 +937,8 @@ __device__ void ib_step_body(const IbArgs<P>& a, int rank, int nranks) {
   }
   ib_phase_final<P, NT>(a, tid, nth, rtid, nband, rank, nranks, red, sh);
   grid_barrier<R>(a.bar, a.ctr, red, a.resid + N, a.cluster, a.bar_limit_ns, nranks);
-  if (rank == 0 && threadIdx.x == 0) ib_check_resid<P>(a);
-  ib_phase_moments<P, NT>(a, tid, nth, rank, nranks, sh);
+  if (rank == 0 && threadIdx.x == 0) ib_check_resid<P>(a, a.resid[a.N]);
+  ib_phase_moments<P, NT>(a, tid, nth, rank, nranks);
   if (a.apply) {
     grid_barrier<R>(a.bar, a.ctr, (const R*)nullptr, (R*)nullptr, a.cluster, a.bar_limit_ns, nranks);
     if (N > 0) ib_phase_apply<P, PAR>(a, tid, nth, nband);   // the apply reads every C_l

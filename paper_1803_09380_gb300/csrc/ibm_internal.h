@@ -102,7 +102,7 @@ struct Ctx {
   void* dent = nullptr;                      // [bcap * kBandCap] Ent<R>, ascending marker id
   void* dbq = nullptr;                       // [bcap][8] band-node quantities (R)
   void* dmq = nullptr;                       // [nm][4] rho*, b (R)
-  void* dAh = nullptr;                       // [n_corr+1][nm][2] momentum deviations A^n (R)
+  void* dAh = nullptr;                       // [n_corr+2][nm][2] momentum deviations A^n (R)
   void* dCm = nullptr;                       // [nm][3] summed second-moment deviation (R)
   void* dG = nullptr;                        // [nm][kGCap] Ent<R> marker coupling rows
   int* dgcnt = nullptr;                      // [nm]
@@ -113,7 +113,7 @@ struct Ctx {
   int* dsegflag = nullptr;                   // [ny][nseg_x] 1 if the segment has a band node
   int* dseglist = nullptr;                   // [segcap] band segments
   BodyDev* dbodies = nullptr;
-  double* dfpart = nullptr;                  // [chunks][nb][3] force partial sums
+  double* dfpart = nullptr;                  // [2][chunks][nb][3] force partial sums
   unsigned long long* dbar = nullptr;        // grid-barrier arrivals of the correction kernel
   int ib_grid = 0;                           // CTAs of the correction kernel
   int ib_grid_max = 0;                       // one per SM
@@ -172,13 +172,13 @@ struct ibm_ctx : public ibm::Ctx {};
 
 namespace ibm {
 
-// Number of CUDA kernels one time step launches (matches enqueue_step).
-inline int kernels_per_step(const Ctx& h) {
+// Number of CUDA kernels one time step launches (matches enqueue_step; timed:
+// with the collide+stream launch bracketed).
+inline int kernels_per_step(const Ctx& h, bool timed = false) {
+  if (h.sl_on && !timed) return 2;                 // the correction, everything else
   int k = 1;                                       // collide + stream
   if (has_nee(h.geom)) k += 1;                     // extrapolation columns
   if (h.nm > 0) {
-    const int N = h.desc.n_corr;
-    (void)N;
     // correction loop (one kernel; one per phase; or pre, cluster, post),
     // band collide+stream
     k += h.ib_phases == 1 ? h.desc.n_corr + 4
@@ -340,6 +340,11 @@ cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s);
 size_t slice_smem(const Ctx& h);
 int slice_max_corr();
 void launch_slice_loop(const Ctx& h, int parity, bool macro, cudaStream_t s);
+// The whole step in two launches on s (the correction, and one kernel for
+// everything else behind it); false: not on slices, or a grid too large.
+// fprev: it also forms the forces and residuals of the step before; fnow: its
+// own (else the next step's launch does).
+bool launch_slice_step(const Ctx& h, int parity, bool macro, bool fprev, bool fnow, cudaStream_t s);
 // Rigid motion of every moving body's markers to its current pose (Eqs. 41-42).
 void launch_marker_move(const Ctx& h, cudaStream_t s);
 

@@ -270,6 +270,14 @@ __device__ __forceinline__ S shfl_up1(S v) { return __shfl_up_sync(0xffffffffu, 
 template <class S>
 __device__ __forceinline__ S shfl_down1(S v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
+// Hides from the compiler that p still has its value: addresses derived from
+// it before are formed anew after, instead of nine of them living in 18
+// registers (and spilling) across the collision.
+template <class T>
+__device__ __forceinline__ void fresh(T*& p) {
+  asm volatile("" : "+l"(p));
+}
+
 // Collide VEC nodes whose pre-collision populations are p[i][k]
 // (arithmetic type), in place, writing macros if asked.
 template <int P, bool MACRO, bool MRT, int VEC>
@@ -322,22 +330,23 @@ __device__ __forceinline__ void even_vec(const Geom& g, const StepConsts<typenam
   typedef typename Prec<P>::S S;
   typedef typename Prec<P>::R R;
   constexpr int VEC = VecTraits<P>::VEC;
-  const long long base = (long long)y * g.nxp + x0;
+  S* at = A + (long long)y * g.nxp + x0;
   R p[9][VEC];
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const SVec<S, VEC> v = vload<S, VEC>(A + i * g.plane + base);
+    const SVec<S, VEC> v = vload<S, VEC>(at + i * g.plane);
 #pragma unroll
     for (int k = 0; k < VEC; ++k) p[i][k] = Prec<P>::ldv(v.v[k], i);
   }
   if (skip) return;
   collide_vec<P, MACRO, MRT, VEC>(g, c, p, mac, x0, y);
+  fresh(at);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     SVec<S, VEC> v;
 #pragma unroll
     for (int k = 0; k < VEC; ++k) v.v[k] = Prec<P>::stv(p[i][k], opp(i));
-    vstore<S, VEC>(A + opp(i) * g.plane + base, v);
+    vstore<S, VEC>(at + opp(i) * g.plane, v);
   }
 }
 
@@ -367,12 +376,13 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
   const bool skip_r = __shfl_down_sync(0xffffffffu, skip, 1);
   const bool lo = lane == 0 || skip_l;                      // left end of an active run
   const bool hi = lane == 31 || skip_r;                     // right end of an active run
+  S* at = A + (long long)y * g.nxp;
+  const long long dm = (long long)(ym - y) * g.nxp, dp = (long long)(yp - y) * g.nxp;
   R p[9][VEC];
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const int sy = cy(i) > 0 ? ym : (cy(i) < 0 ? yp : y);
     const int sl = opp(i);
-    const S* row = A + sl * g.plane + (long long)sy * g.nxp;
+    const S* row = at + sl * g.plane + (cy(i) > 0 ? dm : (cy(i) < 0 ? dp : 0));
     SVec<S, VEC> v;
     if (!skip) {
       v = vload<S, VEC>(row + x0);
@@ -400,10 +410,10 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
   if (sizeof(S) == 2 && full) full_round<VEC>(p);
   collide_vec<P, MACRO, MRT, VEC>(g, c, p, mac, x0, y, !skip);
   if (sizeof(S) == 2 && full) full_round<VEC>(p);
+  fresh(at);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const int ty = cy(i) > 0 ? yp : (cy(i) < 0 ? ym : y);
-    S* row = A + i * g.plane + (long long)ty * g.nxp;
+    S* row = at + i * g.plane + (cy(i) > 0 ? dp : (cy(i) < 0 ? dm : 0));
     S o[VEC];
 #pragma unroll
     for (int k = 0; k < VEC; ++k) o[k] = Prec<P>::stv(p[i][k], i);
@@ -444,6 +454,23 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
       }
     }
   }
+}
+
+// ------------------------------------------------------------------ blocks
+// Threads per collide+stream block (whole warps per row span).  Two warps:
+// a correction-kernel CTA resident beside collide+stream then displaces
+// only the registers it needs, not whole 256-thread blocks (on the 4096^2
+// FP32 Couette step 64 beat 128 and 256 by 0.3 % and 2.4 %; FP16 storage
+// gained 5.6 %; alone the kernel is unchanged).
+constexpr int kK1Threads = 64;
+
+// Resident blocks asked of the register allocator: 1024 threads (64
+// registers) for the node-local even step, 768 (80) for the odd step with
+// its shuffles; FP64 needs 256 threads fewer.  Without it the allocator's
+// own choice varied with unrelated edits, once spilling the odd step's hot
+// loop.
+constexpr int k1_min_blocks(int P, int PAR) {
+  return ((PAR ? 3 : 4) - (P == PREC_FP64 ? 1 : 0)) * (256 / kK1Threads);
 }
 
 // ------------------------------------------------------------------ edges

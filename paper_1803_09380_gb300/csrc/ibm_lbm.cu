@@ -35,22 +35,6 @@ namespace ibm {
 // Even step: per lane, aligned vectors (ragged row ends node by node).  Odd
 // step: the vector path; the first edge_rows rows of blocks take the edge
 // nodes instead, one per thread.
-// Threads per collide+stream block (whole warps per row span).  Two warps:
-// a correction-kernel CTA resident beside collide+stream then displaces
-// only the registers it needs, not whole 256-thread blocks (on the 4096^2
-// FP32 Couette step 64 beat 128 and 256 by 0.3 % and 2.4 %; FP16 storage
-// gained 5.6 %; alone the kernel is unchanged).
-constexpr int kK1Threads = 64;
-
-// Resident blocks asked of the register allocator: 1024 threads (64
-// registers) for the node-local even step, 768 (80) for the odd step with
-// its shuffles; FP64 needs 256 threads fewer.  Without it the allocator's
-// own choice varied with unrelated edits, once spilling the odd step's hot
-// loop.
-constexpr int k1_min_blocks(int P, int PAR) {
-  return ((PAR ? 3 : 4) - (P == PREC_FP64 ? 1 : 0)) * (256 / kK1Threads);
-}
-
 template <int P, int PAR, bool MACRO, int MODE, bool MRT>
 __global__ void __launch_bounds__(kK1Threads, k1_min_blocks(P, PAR)) k_collide_stream(Geom g, StepConsts<typename Prec<P>::R> c,
                                                         typename Prec<P>::S* __restrict__ A,

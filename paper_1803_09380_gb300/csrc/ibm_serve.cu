@@ -106,9 +106,9 @@ double case_bytes(const ibm_lattice_desc& d, int M, int nb) {
   double b = 9.0 * d.ny * nxp * s + 3.0 * nodes * r + 4.0 * nodes + 4.0 * (nxp / 32) * d.ny;
   b += 24.0 * nodes;                                        // staging of rho, ux, uy reads
   b += M * (5 * 8.0 + 4 + 2 * r + 16 * (r + 12) + 4 * r + 3 * r + kGCap * ent + 4);
-  b += M * 2.0 * r * (d.n_corr + 1);
+  b += M * 2.0 * r * (d.n_corr + 2);
   b += bcap * (8 + kBandCap * ent + 8 * r + 4);
-  b += nb * (sizeof(ibm::BodyDev) + 24.0 * (M / kForceChunk + 1));
+  b += nb * (sizeof(ibm::BodyDev) + 48.0 * (M / kForceChunk + 1));
   return b + (1 << 20) + 2.0 * (16 << 20);                  // + the unused part of two 16 MiB chunks
 }
 

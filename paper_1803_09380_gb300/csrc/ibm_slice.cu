@@ -251,7 +251,8 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
   R* rso = dv + kStencil * LM;                                                  // [SM] rho* of the owned markers
   R* sew = rso + SM;                          // [EM][X1M] covering lists
   int* sen = reinterpret_cast<int*>(sew + (size_t)EM * X1M);
-  unsigned short* sei = reinterpret_cast<unsigned short*>(sen + X1M);
+  int* sbid = sen + X1M;                                     // [X1M] band indices of the owned nodes
+  unsigned short* sei = reinterpret_cast<unsigned short*>(sbid + X1M);
   unsigned short* dk = sei + (size_t)EM * X1M;               // [kStencil][LM] their nodes
   __shared__ typename AtomicBits<R>::U rmax[kSliceMaxCorr + 2];   // residual maxima, as bits
   __shared__ int depth[kSliceMaxCorr + 2];                   // markers of depth <= h
@@ -260,6 +261,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
   const int nown = head[0], nX1 = head[1], nX = head[2];
   const int own = head[4], nloc = head[4 + N], d1 = head[5];
   const size_t sm = (size_t)s * kSliceMarkers;
+  dependency_release();                                      // k_slice_stream starts beside this kernel
 #pragma unroll 1
   for (int k = t; k <= N; k += NT) {
     depth[k] = head[4 + k];
@@ -298,9 +300,10 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
     }
   }
   {
-    // a row of the lists per warp: EM of weights, EM of markers, the counts
+    // a row of the lists per warp: EM of weights, EM of markers, the counts,
+    // the band indices
 #pragma unroll 1
-    for (int j = t >> 5; j <= 2 * EM; j += NT / 32) {
+    for (int j = t >> 5; j <= 2 * EM + 1; j += NT / 32) {
       const char* from;
       char* to;
       int bytes;
@@ -313,9 +316,9 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
         to = (char*)(sei + (size_t)(j - EM) * X1M);
         bytes = nX1 * (int)sizeof(short);
       } else {
-        from = (const char*)(sl.en + (size_t)s * kSliceX1);
-        to = (char*)sen;
-        bytes = nX1 * (int)sizeof(int);
+        from = (const char*)((j == 2 * EM ? sl.en : sl.bid) + (size_t)s * kSliceX1);
+        to = (char*)(j == 2 * EM ? sen : sbid);
+        bytes = (j == 2 * EM ? nX1 : nown) * (int)sizeof(int);
       }
 #pragma unroll 1
       for (int k = (t & 31) * 16; k < bytes; k += 512) copy16_async(to + k, from + k);
@@ -324,14 +327,15 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
   R w[kStencil];
   unsigned int wi[kStencil / 2];
   R ux = R(0), uy = R(0);
+  int mid = 0;
   if (t < nloc) {
 #pragma unroll
     for (int q = 0; q < kStencil; ++q) w[q] = sl.w[((size_t)s * kStencil + q) * kSliceMarkers + t];
 #pragma unroll
     for (int q = 0; q < kStencil / 2; ++q) wi[q] = sl.wi[((size_t)s * (kStencil / 2) + q) * kSliceMarkers + t];
-    const int m = sl.mid[sm + t];
-    ux = a.Ux[m];
-    uy = a.Uy[m];
+    mid = sl.mid[sm + t];
+    ux = a.Ux[mid];
+    uy = a.Uy[mid];
   }
   R rw[kRowHead];
   unsigned short ri[kRowHead];
@@ -345,6 +349,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
       ri[j] = sl.ri[((size_t)s * kSliceRow + j) * kSliceMarkers + t];
     }
   }
+  copy_async_wait();
   __syncthreads();
 
   // rho*, J*^0, b = A^1 (Eq. 22b, Eq. 28 in moment form)
@@ -412,7 +417,6 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
         hist[(size_t)(n + 1) * LM + t] = v;
       }
     }
-    if (n == N) copy_async_wait();
     __syncthreads();
   }
 
@@ -472,7 +476,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
   for (int k = t; k < nX1; k += NT) {
     const R j0x = njx[k], j0y = njy[k];
     R axx = R(0), axy = R(0), ayy = R(0);
-    R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
+    R* o = a.bq + 8 * (long long)sbid[k < nown ? k : 0];
     if (F64) {
 #pragma unroll 1
       for (int n = 0; n < N; ++n) {
@@ -548,11 +552,11 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
     V v;
     v.x = ax;
     v.y = ay;
-    reinterpret_cast<V*>(a.Ah)[(long long)N * a.M + sl.mid[sm + t]] = v;
+    reinterpret_cast<V*>(a.Ah)[(long long)(N + PAR) * a.M + mid] = v;
   }
 #pragma unroll 1
   for (int n = t; n <= N; n += NT)
-    sl.rpart[(size_t)s * (kSliceMaxCorr + 2) + n] = AtomicBits<R>::from_bits(rmax[n]);
+    sl.rpart[((size_t)PAR * sl.count + s) * (kSliceMaxCorr + 2) + n] = AtomicBits<R>::from_bits(rmax[n]);
   __syncthreads();
 
   // Eq. 27 summed: the second-moment correction of the owned nodes
@@ -568,7 +572,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
       pxy += wj * cm[LM + m];
       pyy += wj * cm[2 * LM + m];
     }
-    R* o = a.bq + 8 * (long long)sl.bid[(size_t)s * kSliceX1 + k];
+    R* o = a.bq + 8 * (long long)sbid[k];
     o[3] = pxx;
     o[4] = pxy;
     o[5] = pyy;
@@ -582,7 +586,8 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
 // overwrites all nine slots that it reads, so the corrected populations stay
 // in registers (rounded as the storage rounds them).  Nodes on a closed or
 // open side go through the boundary rules.
-template <int P, int PAR, bool MACRO, bool MRT>
+// WAIT: the correction comes from the kernel launched before.
+template <int P, int PAR, bool MACRO, bool MRT, bool WAIT>
 __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
   typedef typename Prec<P>::R R;
   typedef typename Prec<P>::S S;
@@ -590,6 +595,7 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
   S* __restrict__ A = a.A;
   const int b = a.node2band[y * g.nx + x];
   if (PAR == 1 && needs_boundary_path(g, x, y)) {
+    if (WAIT) dependency_wait();
     if (b >= 0) {
       const R* q = a.bq + 8 * (long long)b;
 #pragma unroll
@@ -613,6 +619,7 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
     const int sy = PAR == 0 ? y : (cy(i) > 0 ? ym : (cy(i) < 0 ? yp : y));
     v[i] = A[(PAR == 0 ? i : opp(i)) * g.plane + (long long)sy * g.nxp + sx];
   }
+  if (WAIT) dependency_wait();
   R p[9], ps[9], rho, jx, jy;
 #pragma unroll
   for (int i = 0; i < 9; ++i) p[i] = Prec<P>::ld(v[i], PAR == 0 ? i : opp(i));
@@ -642,62 +649,142 @@ __device__ __forceinline__ void finish_node(const IbArgs<P>& a, int x, int y) {
   }
 }
 
-// Block 0 reduces the slices' residual maxima, the next nchunk blocks form
-// the body forces (one chunk of kForceChunk markers each; the last to arrive
-// adds the chunks up), the others collide and stream the 32-node row segments
-// that hold band nodes, one warp per segment.  The forces are the longest
-// chain in it: with one trip of loads per chunk, a halving tree for the FP64
-// sums and the residuals in a block of their own it takes 10.8 us instead of
-// 20.4 on a 300^2 lattice with 1029 markers (cold caches).
-constexpr int kFinishThreads = kForceChunk;
-template <int P, int PAR, bool MACRO, bool MRT>
-__global__ void __launch_bounds__(kFinishThreads) k_band_finish(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
+// The residuals and body forces of the step whose correction ran with parity
+// `par`, by block k0 of 1 + nchunk blocks of NT threads: block 0 reduces the
+// slices' residual maxima, the others form the forces, one chunk of kForceChunk
+// markers each; the last to arrive adds the chunks up.  WAIT: that correction
+// is the kernel launched before (what does not depend on it is loaded before
+// the wait).  store false: a later step's results, formed in the same launch,
+// are the ones to keep.
+template <int P, int NT, bool WAIT>
+__device__ __forceinline__ void force_block(const IbArgs<P>& a, const SliceArgs<typename Prec<P>::R>& sl, int k0,
+                                            int par, bool store, ForceShared<NT>& sh) {
   typedef typename Prec<P>::R R;
-  const int nchunk = (a.M + kForceChunk - 1) / kForceChunk, nfin = nchunk + 1;
-  if (blockIdx.x == 0) {
+  const int nchunk = (a.M + kForceChunk - 1) / kForceChunk;
+  if (k0 == 0) {
+    if (WAIT) dependency_wait();
     const int lane = threadIdx.x & 31;
+    const R* rp = sl.rpart + (size_t)par * sl.count * (kSliceMaxCorr + 2);
 #pragma unroll 1
-    for (int n = threadIdx.x >> 5; n <= a.N; n += kFinishThreads / 32) {
+    for (int n = threadIdx.x >> 5; n <= a.N; n += NT / 32) {
       R m = R(0);
-      for (int k = lane; k < sl.count; k += 32) m = nanmax(m, sl.rpart[(size_t)k * (kSliceMaxCorr + 2) + n]);
+      for (int k = lane; k < sl.count; k += 32) m = nanmax(m, rp[(size_t)k * (kSliceMaxCorr + 2) + n]);
 #pragma unroll
       for (int off = 16; off >= 1; off >>= 1) m = nanmax(m, __shfl_xor_sync(0xffffffffu, m, off));
       if (lane == 0) {
-        a.resid[n] = m;
-        if (n == a.N) ib_check_resid<P>(a);
+        if (store) a.resid[n] = m;
+        if (n == a.N) ib_check_resid<P>(a, m);
       }
     }
     return;
   }
-  if ((int)blockIdx.x < nfin) {
-    __shared__ double sh[kChunkSumShared];
-    __shared__ int last;
-    ib_force_chunk<P>(a, a.Ah + (long long)a.N * 2 * a.M, blockIdx.x - 1, sh);
-    if (nchunk > 1) {
-      if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(sl.fin, 1) == nchunk - 1;
-        if (last) *sl.fin = 0;                             // the next launch starts from zero
-        __threadfence();
-      }
-      __syncthreads();
-      if (!last) return;
+  double* fpart = a.fpart + (size_t)par * nchunk * a.nb * 3;
+  ib_force_chunk<P, NT, WAIT>(a, a.Ah + (long long)(a.N + par) * 2 * a.M, k0 - 1, fpart, sh);
+  if (nchunk > 1) {
+    if (threadIdx.x == 0) {
+      __threadfence();
+      sh.last = atomicAdd(sl.fin + par, 1) == nchunk - 1;
+      if (sh.last) sl.fin[par] = 0;                           // the next launch starts from zero
+      __threadfence();
     }
-    ib_force_total<P>(a, 0, 1);
-    return;
+    __syncthreads();
+    if (!sh.last) return;
   }
+  ib_force_total<P>(a, 0, 1, fpart, store);
+}
+
+// The 32-node row segments that hold band nodes, collided and streamed, one
+// warp per segment, by block k0 of nblk.  WAIT: as above; the segments'
+// populations are loaded before the wait.
+template <int P, int PAR, bool MACRO, bool MRT, int NT, bool WAIT>
+__device__ __forceinline__ void band_block(const IbArgs<P>& a, int k0, int nblk) {
   const Geom& g = a.g;
   const int nseg = a.ctr[CTR_NSEG];
   const int lane = threadIdx.x & (kSegW - 1);
   // blocks first, then their warps: few segments spread over all SMs
-  const int nblk = gridDim.x - nfin;
 #pragma unroll 1
-  for (int k = (threadIdx.x >> 5) * nblk + blockIdx.x - nfin; k < nseg; k += nblk * (kFinishThreads / 32)) {
+  for (int k = (threadIdx.x >> 5) * nblk + k0; k < nseg; k += nblk * (NT / 32)) {
     const int seg = a.seglist[k];
     const int y = seg / a.nseg_x, x = (seg - y * a.nseg_x) * kSegW + lane;
-    if (x >= g.nx || nee_column(g, x)) continue;          // k_open_columns streams those
-    finish_node<P, PAR, MACRO, MRT>(a, x, y);
+    if (x >= g.nx || nee_column(g, x)) continue;          // the extrapolation columns are streamed apart
+    finish_node<P, PAR, MACRO, MRT, WAIT>(a, x, y);
   }
+}
+
+constexpr int kFinishThreads = kForceChunk;
+template <int P, int PAR, bool MACRO, bool MRT>
+__global__ void __launch_bounds__(kFinishThreads) k_band_finish(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
+  const int nfin = 1 + (a.M + kForceChunk - 1) / kForceChunk;
+  __shared__ ForceShared<kFinishThreads> fs;
+  if ((int)blockIdx.x < nfin) force_block<P, kFinishThreads, false>(a, sl, blockIdx.x, PAR, true, fs);
+  else band_block<P, PAR, MACRO, MRT, kFinishThreads, false>(a, blockIdx.x - nfin, gridDim.x - nfin);
+}
+
+// Everything of a step but the correction, as one launch behind the slice
+// kernel (programmatic dependent launch): rows of blocks with the edge nodes
+// (odd step), the band-free spans and the extrapolation columns, which need
+// nothing of the correction and run beside it, then the band segments, which
+// wait for it.  Those come after three quarters of the lattice's rows: on a
+// large lattice they then find the correction done (20 us into the 175 to 190
+// us of a 4096^2 FP32 step) instead of holding registers while they wait, and
+// are not the launch's tail, where their dependent loads took 10 us.  The
+// correction releases this launch at its start: released after its gather, it
+// ended earlier (17 against 21 us) but the step later (188 and 204 us, even
+// and odd, against 185 and 201).  One stream and two launches a step, without
+// fork, join or priorities.
+//
+// The forces are the longest chain behind the correction (5 us against 1.5
+// for the band: two dependent FP64 sums with an arrival between them), so
+// inside a graph of several steps each step's forces and residuals are formed
+// in the next step's launch, off the chain; the graph's last step forms its own.
+struct StepShape {
+  int bx;                      // blocks per row
+  int edge_rows, span_rows;    // rows of blocks: edge nodes, lattice rows
+  int head_rows, tail_rows;    // lattice rows before the rows of the blocks below; those
+  int open;                    // blocks of extrapolation columns,
+  int fprev, fnow;             // of the previous and this step's forces (0: none),
+  int nblk;                    // and of band segments
+};
+constexpr int kStepThreads = kK1Threads;
+template <int P, int PAR, bool MACRO, bool MRT>
+__global__ void __launch_bounds__(kStepThreads, k1_min_blocks(P, PAR))
+    k_slice_stream(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl, const int* __restrict__ segflag, StepShape sh) {
+  __shared__ ForceShared<kStepThreads> fs;
+  int row = blockIdx.y;
+  if (PAR == 1) {
+    if (row < sh.edge_rows) {
+      k1_edge_node<P, MACRO, K1_MAIN, MRT>(a.g, a.c, a.A, a.mac, segflag, a.nseg_x,
+                                           ((long long)row * sh.bx + blockIdx.x) * kStepThreads + threadIdx.x);
+      return;
+    }
+    row -= sh.edge_rows;
+  }
+  const bool tail = row >= sh.head_rows && row < sh.head_rows + sh.tail_rows;
+  if (!tail) {
+    if (row >= sh.head_rows) row -= sh.tail_rows;
+    k1_span<P, PAR, MACRO, K1_MAIN, MRT>(a.g, a.c, a.A, a.mac, segflag, a.nseg_x, row,
+                                         (blockIdx.x * kStepThreads + threadIdx.x) >> 5, threadIdx.x & 31);
+    return;
+  }
+  int k = (row - sh.head_rows) * sh.bx + blockIdx.x;
+  if (k < sh.open) {
+    const int q = k * kStepThreads + threadIdx.x;
+    if (q < 2 * a.g.ny) open_column<P, PAR, MACRO, MRT>(a.g, a.c, a.A, a.mac, q / a.g.ny, q % a.g.ny);
+    return;
+  }
+  k -= sh.open;
+  if (k < sh.fprev) {
+    force_block<P, kStepThreads, false>(a, sl, k, PAR ^ 1, sh.fnow == 0, fs);
+    return;
+  }
+  k -= sh.fprev;
+  if (k < sh.fnow) {
+    force_block<P, kStepThreads, true>(a, sl, k, PAR, true, fs);
+    return;
+  }
+  k -= sh.fnow;
+  if (k == 0) dependency_wait();                           // the launch ends after the correction in any case
+  if (k < sh.nblk) band_block<P, PAR, MACRO, MRT, kStepThreads, true>(a, k, sh.nblk);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -724,7 +811,7 @@ size_t slice_mem_bytes(int prec, int count) {
 template <class R>
 static cudaError_t slice_build_t(const Ctx& h, int* stat, cudaStream_t s) {
   SliceArgs<R> a = slice_args<R>(h);
-  cudaError_t e = cudaMemsetAsync(a.fin, 0, sizeof(int), s);
+  cudaError_t e = cudaMemsetAsync(a.fin, 0, 2 * sizeof(int), s);
   if (e != cudaSuccess) return e;
   k_slice_build<R><<<h.sl_count, kSliceThreads, 0, s>>>(a, h.nm, h.desc.n_corr, h.dctr, h.dband_of, (const R*)h.dW,
                                                         h.dbnode, h.dbcnt, (const Ent<R>*)h.dent,
@@ -736,6 +823,13 @@ cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s) {
   return h.r_bytes == 8 ? slice_build_t<double>(h, stat, s) : slice_build_t<float>(h, stat, s);
 }
 
+// Share of an SM's memory that both kernels of a step ask for as shared memory
+// (100 KB), so that their blocks can be resident together: the correction
+// takes 45 to 95 KB, and with each kernel's own choice of the split the 4096^2
+// FP32 step took 206 us instead of 200 (at 72 % and more the loss of L1 cost
+// as much).
+constexpr int kStepCarveout = 44;
+
 // Shared memory of the slice kernel for the planned slices, or 0 when the
 // device cannot give it.
 template <int P>
@@ -744,8 +838,25 @@ static size_t slice_smem_t(const Ctx& h) {
                                                             h.desc.n_corr);
   constexpr size_t kMax = 200 * 1024;
   if (need > kMax) return 0;
-  if (cudaFuncSetAttribute(k_ib_slice<P, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax) != cudaSuccess ||
-      cudaFuncSetAttribute(k_ib_slice<P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax) != cudaSuccess) {
+  bool ok = true;
+  auto set = [&](auto kern, bool slice) {
+    if (slice) ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, kStepCarveout) == cudaSuccess;
+  };
+  set(k_ib_slice<P, 0>, true);
+  set(k_ib_slice<P, 1>, true);
+  if (h.desc.collision == IBM_COLL_MRT) {
+    set(k_slice_stream<P, 0, false, true>, false);
+    set(k_slice_stream<P, 0, true, true>, false);
+    set(k_slice_stream<P, 1, false, true>, false);
+    set(k_slice_stream<P, 1, true, true>, false);
+  } else {
+    set(k_slice_stream<P, 0, false, false>, false);
+    set(k_slice_stream<P, 0, true, false>, false);
+    set(k_slice_stream<P, 1, false, false>, false);
+    set(k_slice_stream<P, 1, true, false>, false);
+  }
+  if (!ok) {
     cudaGetLastError();
     return 0;
   }
@@ -762,14 +873,21 @@ size_t slice_smem(const Ctx& h) {
 }
 
 template <int P>
-static void slice_loop_t(const Ctx& h, int parity, bool macro, cudaStream_t s) {
+static void launch_slices(const Ctx& h, int parity, cudaStream_t s, const IbArgs<P>& a,
+                          const SliceArgs<typename Prec<P>::R>& sl) {
   typedef typename Prec<P>::R R;
-  IbArgs<P> a = make_ib_args<P>(h);
-  SliceArgs<R> sl = slice_args<R>(h);
   const size_t smem = slice_smem_bytes<R>(sl.xmax, sl.x1max, sl.lmax, sl.emax, sl.S, a.N);
   const dim3 grid(sl.count), block(kSliceThreads);
   if (parity == 0) launch_prio_smem(k_ib_slice<P, 0>, grid, block, smem, s, h.ib_prio, a, sl);
   else launch_prio_smem(k_ib_slice<P, 1>, grid, block, smem, s, h.ib_prio, a, sl);
+}
+
+template <int P>
+static void slice_loop_t(const Ctx& h, int parity, bool macro, cudaStream_t s) {
+  typedef typename Prec<P>::R R;
+  IbArgs<P> a = make_ib_args<P>(h);
+  SliceArgs<R> sl = slice_args<R>(h);
+  launch_slices<P>(h, parity, s, a, sl);
   const int nchunk = (h.nm + kForceChunk - 1) / kForceChunk;
   const dim3 g2(1 + nchunk + std::max(1, std::min(h.sl_nseg, 16 * h.ib_grid_max))), b2(kFinishThreads);
   auto go = [&](auto kern) { launch_prio(kern, g2, b2, s, h.ib_prio, a, sl); };
@@ -779,6 +897,72 @@ static void slice_loop_t(const Ctx& h, int parity, bool macro, cudaStream_t s) {
   } else {
     if (parity == 0) { if (macro) go(k_band_finish<P, 0, true, false>); else go(k_band_finish<P, 0, false, false>); }
     else { if (macro) go(k_band_finish<P, 1, true, false>); else go(k_band_finish<P, 1, false, false>); }
+  }
+}
+
+// Grid of k_slice_stream; bx = 0 when it does not fit a launch.
+template <int P, int PAR>
+static StepShape step_shape(const Ctx& h, bool fprev, bool fnow) {
+  constexpr int VEC = PAR ? VecTraits<P>::VEC_ODD : VecTraits<P>::VEC;
+  const Geom& g = h.geom;
+  StepShape sh;
+  sh.bx = ((g.nx + 32 * VEC - 1) / (32 * VEC) + kStepThreads / 32 - 1) / (kStepThreads / 32);
+  const long long per_row = (long long)sh.bx * kStepThreads;
+  const long long edge = PAR ? edge_nodes(g, odd_edge<VEC>(g)) : 0;
+  sh.edge_rows = (int)((edge + per_row - 1) / per_row);
+  sh.span_rows = g.ny;
+  sh.open = has_nee(g) ? (2 * g.ny + kStepThreads - 1) / kStepThreads : 0;
+  const int nfin = 1 + (h.nm + kForceChunk - 1) / kForceChunk;
+  sh.fprev = fprev ? nfin : 0;
+  sh.fnow = fnow ? nfin : 0;
+  // a segment per block while that fills the SMs, then one per warp
+  sh.nblk = std::max({1, std::min(h.sl_nseg, 16 * h.ib_grid_max), (h.sl_nseg + kStepThreads / 32 - 1) / (kStepThreads / 32)});
+  sh.head_rows = g.ny - g.ny / 4;
+  sh.tail_rows = (int)(((long long)sh.open + sh.fprev + sh.fnow + sh.nblk + sh.bx - 1) / sh.bx);
+  return sh;
+}
+static long long step_rows(const StepShape& sh) { return (long long)sh.edge_rows + sh.span_rows + sh.tail_rows; }
+
+template <int P, int PAR, bool MACRO, bool MRT>
+static void launch_stream(const Ctx& h, cudaStream_t s, const IbArgs<P>& a,
+                          const SliceArgs<typename Prec<P>::R>& sl, bool fprev, bool fnow) {
+  const StepShape sh = step_shape<P, PAR>(h, fprev, fnow);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(sh.bx, (unsigned)step_rows(sh));
+  cfg.blockDim = dim3(kStepThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_slice_stream<P, PAR, MACRO, MRT>, a, sl, (const int*)h.dsegflag, sh);
+}
+
+template <int P>
+static bool slice_step_t(const Ctx& h, int parity, bool macro, bool fprev, bool fnow, cudaStream_t s) {
+  // the same answer for every step of the lattice
+  if (step_rows(step_shape<P, 1>(h, true, true)) > 65535) return false;
+  IbArgs<P> a = make_ib_args<P>(h);
+  SliceArgs<typename Prec<P>::R> sl = slice_args<typename Prec<P>::R>(h);
+  launch_slices<P>(h, parity, s, a, sl);
+  if (a.c.mrt) {
+    if (parity == 0) { if (macro) launch_stream<P, 0, true, true>(h, s, a, sl, fprev, fnow); else launch_stream<P, 0, false, true>(h, s, a, sl, fprev, fnow); }
+    else { if (macro) launch_stream<P, 1, true, true>(h, s, a, sl, fprev, fnow); else launch_stream<P, 1, false, true>(h, s, a, sl, fprev, fnow); }
+  } else {
+    if (parity == 0) { if (macro) launch_stream<P, 0, true, false>(h, s, a, sl, fprev, fnow); else launch_stream<P, 0, false, false>(h, s, a, sl, fprev, fnow); }
+    else { if (macro) launch_stream<P, 1, true, false>(h, s, a, sl, fprev, fnow); else launch_stream<P, 1, false, false>(h, s, a, sl, fprev, fnow); }
+  }
+  return true;
+}
+
+bool launch_slice_step(const Ctx& h, int parity, bool macro, bool fprev, bool fnow, cudaStream_t s) {
+  if (!h.sl_on) return false;
+  switch (h.prec) {
+    case PREC_FP64: return slice_step_t<PREC_FP64>(h, parity, macro, fprev, fnow, s);
+    case PREC_FP32: return slice_step_t<PREC_FP32>(h, parity, macro, fprev, fnow, s);
+    case PREC_FP16_DEV: return slice_step_t<PREC_FP16_DEV>(h, parity, macro, fprev, fnow, s);
+    default: return slice_step_t<PREC_BF16_DEV>(h, parity, macro, fprev, fnow, s);
   }
 }
 

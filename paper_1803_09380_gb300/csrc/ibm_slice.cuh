@@ -17,9 +17,9 @@
 // whatever the slices.
 //
 // Measured against the persistent kernel with its band collide (us per step,
-// whole steps): 300^2 FP32 with 1029 markers 68.1 -> 30.5, 1024^2 FP32 with
-// 3513 markers 72.3 -> 36.1, 4096^2 FP32 with 14052 markers beside
-// collide+stream 220.8 -> 203.0, 64^2 FP64 with 220 markers 204.1 -> 67.5.
+// whole steps): 300^2 FP32 with 1029 markers 68.1 -> 16.4, 1024^2 FP32 with
+// 3513 markers 72.3 -> 21.6, 4096^2 FP32 with 14052 markers beside
+// collide+stream 220.8 -> 202.4, 64^2 FP64 with 220 markers 204.1 -> 39.0.
 //
 // What bounds it: latency.  The persistent kernel paid thirteen grid
 // barriers, each followed by dependent loads from L2; here the only global
@@ -67,8 +67,8 @@ struct SliceArgs {
   int* en;                     // [count][kSliceX1] covering markers of a node
   R* ew;                       // [count][kSliceEnt][kSliceX1] W_l ds_l
   unsigned short* ei;          // [count][kSliceEnt][kSliceX1] local markers
-  R* rpart;                    // [count][kSliceMaxCorr + 2] the slices' residual maxima
-  int* fin;                    // arrivals of the force chunks; zero between launches
+  R* rpart;                    // [2][count][kSliceMaxCorr + 2] the slices' residual maxima, by step parity
+  int* fin;                    // [2] arrivals of the force chunks; zero between launches
 };
 
 // Device bytes of `count` slices, and the pieces of that block.
@@ -82,7 +82,7 @@ inline size_t slice_bytes(int count, unsigned char* base, SliceArgs<R>* s) {
   };
   const size_t n = (size_t)count;
   SliceArgs<R> t{};
-  t.fin = (int*)take(sizeof(int));
+  t.fin = (int*)take(2 * sizeof(int));
   t.head = (int*)take(n * kSliceHead * sizeof(int));
   t.mid = (int*)take(n * kSliceMarkers * sizeof(int));
   t.nid = (int*)take(n * kSliceNodes * sizeof(int));
@@ -95,7 +95,7 @@ inline size_t slice_bytes(int count, unsigned char* base, SliceArgs<R>* s) {
   t.en = (int*)take(n * kSliceX1 * sizeof(int));
   t.ew = (R*)take(n * kSliceEnt * kSliceX1 * sizeof(R));
   t.ei = (unsigned short*)take(n * kSliceEnt * kSliceX1 * sizeof(short));
-  t.rpart = (R*)take(n * (kSliceMaxCorr + 2) * sizeof(R));
+  t.rpart = (R*)take(2 * n * (kSliceMaxCorr + 2) * sizeof(R));
   if (s) {
     t.count = s->count; t.S = s->S; t.xmax = s->xmax; t.x1max = s->x1max;
     t.lmax = s->lmax; t.emax = s->emax;
@@ -107,12 +107,13 @@ inline size_t slice_bytes(int count, unsigned char* base, SliceArgs<R>* s) {
 // Dynamic shared memory of one slice CTA, in the order of its pieces: the A
 // history, the owned markers' dj^n, (FP64) j^n of the depth <= 1 markers'
 // nodes; rho, j of the nodes; sum_n j^n j^n; C; W / rho; rho* of the owned
-// markers; the covering lists' weights, counts and markers; the nodes of W / rho.
+// markers; the covering lists' weights and counts, the band indices, the
+// lists' markers; the nodes of W / rho.
 template <class R>
 __host__ __device__ constexpr size_t slice_smem_bytes(int xmax, int x1max, int lmax, int emax, int S, int N) {
   return 2 * sizeof(R) * ((size_t)(N + 1) * (lmax + ((S + 3) & ~3)) + (sizeof(R) == 8 ? (size_t)(N + 1) * x1max : 0)) +
          sizeof(R) * ((size_t)3 * xmax + (size_t)3 * x1max + (size_t)3 * lmax + ((S + 3) & ~3)) +
-         (size_t)emax * x1max * (sizeof(R) + sizeof(short)) + (size_t)x1max * sizeof(int) +
+         (size_t)emax * x1max * (sizeof(R) + sizeof(short)) + (size_t)x1max * 2 * sizeof(int) +
          (size_t)kStencil * lmax * (sizeof(R) + sizeof(short));
 }
 
