@@ -189,7 +189,8 @@ void enqueue_step(Ctx& h, int parity, bool macro, bool timing, bool fprev, bool 
     if (t) cudaEventRecord(e[0], h.stream);
     launch_collide_stream(h, parity, macro, K1_ALL, h.stream);
     if (t) cudaEventRecord(e[1], h.stream);
-  } else if (!timing && launch_slice_step(h, parity, macro, fprev, fnow, h.stream)) {
+  } else if (!timing && launch_slice_step(h, parity, macro, fprev && !h.any_moving, fnow || h.any_moving, h.stream)) {
+    launch_body_update(h, h.stream);
   } else {
     cudaEventRecord(h.ev_fork, h.stream);
     cudaStreamWaitEvent(h.ib_stream, h.ev_fork, 0);
@@ -278,8 +279,9 @@ int slice_size(const Ctx& c) {
 }
 
 // Plans the barrier-free correction for the current band: builds the slices'
-// lists, halving the slices while one does not fit.  Without it (moving
-// bodies, another launch form asked for, markers too dense for any slice, no
+// lists, halving the slices while one does not fit; moving bodies of up to 256
+// markers run on one slice that is rebuilt every step.  Without it (more
+// moving markers, another launch form asked for, markers too dense for any slice, no
 // memory) steps run the persistent kernel.  Synchronises the stream once
 // per attempt; a stream that is being captured is left alone.
 void plan_slices(Ctx& c) {
@@ -289,9 +291,23 @@ void plan_slices(Ctx& c) {
     return;
   }
   c.sl_tried = true;
-  if (c.nm == 0 || c.any_moving || !c.band_collide || c.ib_phases != 0 || c.ib_threads != kIbThreads ||
+  if (c.nm == 0 || !c.band_collide || c.ib_phases != 0 || c.ib_threads != kIbThreads ||
       c.test_drop_arrival || c.desc.n_corr < 1 || c.desc.n_corr > slice_max_corr())
     return;
+  if (c.any_moving) {
+    if (c.ib_grid_opt > 1 || !slice_moving_fits(c)) return;
+    c.sl_mem = dev_alloc(c, slice_mem_bytes(c.prec, 1));
+    if (!c.sl_mem) return;
+    if (cudaMemsetAsync(c.sl_mem, 0, slice_mem_bytes(c.prec, 1), c.stream) != cudaSuccess ||
+        launch_rebuild(c, false, c.stream) != cudaSuccess) {
+      cudaGetLastError();
+      dev_free(c, c.sl_mem);
+      c.sl_mem = nullptr;
+      return;
+    }
+    c.sl_on = true;
+    return;
+  }
   if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 8 * sizeof(int)))) return;
   const int asked = c.ib_grid_opt > 0 ? (c.nm + c.ib_grid - 1) / c.ib_grid : 0;
   for (int S = asked ? asked : slice_size(c); S >= 1; S /= 2) {
@@ -328,10 +344,18 @@ void plan_slices(Ctx& c) {
 // Forgets the slices (the band, or an option that they depend on, changes);
 // the caller has synchronised the stream and drops the graphs.
 void drop_slices(Ctx& c) {
+  if (c.sl_on && c.any_moving) c.band_valid = false;   // its rebuild leaves out the general path's lists
   if (c.sl_mem) dev_free(c, c.sl_mem);
   c.sl_mem = nullptr;
   c.sl_on = c.sl_tried = false;
   c.sl_count = 0;
+}
+
+// The band of the current marker positions.
+void build_band(Ctx& c) {
+  if (c.sl_on && c.any_moving) launch_rebuild(c, false, c.stream);
+  else launch_band_build(c, c.stream);
+  c.band_valid = true;
 }
 
 ibm_status upload_markers(Ctx* h) {
@@ -760,8 +784,7 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
       for (auto& e : c.ev) IBM_CK(h, cudaEventCreate(&e));
     }
     if (c.nm > 0 && !c.band_valid) {
-      launch_band_build(c, c.stream);
-      c.band_valid = true;
+      build_band(c);
       if (c.ib_phases == 1) {
         ibm_status st = count_band(h);
         if (st != IBM_OK) return st;
@@ -1051,8 +1074,7 @@ ibm_status ibm_get_sizes(ibm_handle h, long long* nodes, int* markers, int* bodi
   if (band_nodes || band_segments) {
     int ctr[CTR_COUNT] = {0, 0, 0, 0};
     if (h->nm > 0 && !h->band_valid) {
-      launch_band_build(*h, h->stream);
-      h->band_valid = true;
+      build_band(*h);
     }
     IBM_CK(h, cudaMemcpyAsync(ctr, h->dctr, sizeof(ctr), cudaMemcpyDeviceToHost, h->stream));
     IBM_CK(h, cudaStreamSynchronize(h->stream));

@@ -629,6 +629,10 @@ static void body_update_t(const Ctx& h, cudaStream_t s) {
 
 void launch_body_update(const Ctx& h, cudaStream_t s) {
   if (h.nb == 0 || !h.any_moving) return;
+  if (h.sl_on) {
+    launch_rebuild(h, true, s);
+    return;
+  }
   if (h.r_bytes == 8) body_update_t<double>(h, s);
   else body_update_t<float>(h, s);
 }

@@ -949,10 +949,10 @@ __device__ void ib_step_body(const IbArgs<P>& a, int rank, int nranks) {
 // Eq. 39 on body i from a partner at offset d = x_i - x_j.
 __device__ inline void collision_force(const BodyDev& Bi, double Rj, double dx, double dy, double* F) {
   const double eps_c = 0.01, xi = 0.05 * 2.0 * Bi.radius;
-  const double gmag = sqrt(Bi.gravity[0] * Bi.gravity[0] + Bi.gravity[1] * Bi.gravity[1]);
-  const double cij = Bi.mass * (1.0 - Bi.rho_f / Bi.rho_s) * gmag;
   const double d = sqrt(dx * dx + dy * dy);
   if (d > Bi.radius + Rj + xi || d <= 0.0) return;
+  const double gmag = sqrt(Bi.gravity[0] * Bi.gravity[0] + Bi.gravity[1] * Bi.gravity[1]);
+  const double cij = Bi.mass * (1.0 - Bi.rho_f / Bi.rho_s) * gmag;
   const double s = (d - Bi.radius - Rj - xi) / xi;
   F[0] += cij / eps_c * s * s * dx / d;
   F[1] += cij / eps_c * s * s * dy / d;
@@ -962,24 +962,50 @@ __device__ inline void collision_force(const BodyDev& Bi, double Rj, double dx, 
 // blockDim.x, FP64): Eqs. 37-38 (internal-mass terms, lagged), 39
 // (collisions with other free bodies and with mirror images across closed
 // walls), 40-42.  Every thread of the CTA calls it (it holds a block barrier).
+constexpr int kPairBodies = 8;   // up to this many bodies: a thread per partner
 __device__ inline void body_update_cta(const Geom& g, BodyDev* __restrict__ bodies, int nb) {
   const int b = threadIdx.x;
   double Fc[2] = {0.0, 0.0};
   BodyDev B;
-  if (b < nb) {
-    B = bodies[b];
-    if (B.kind == IBM_BODY_FREE) {
-      for (int o = 0; o < nb; ++o) {
-        if (o == b || bodies[o].kind != IBM_BODY_FREE) continue;
-        collision_force(B, bodies[o].radius, B.xc[0] - bodies[o].xc[0], B.xc[1] - bodies[o].xc[1], Fc);
-      }
-      for (int s = 0; s < 4; ++s) {
-        if (g.bc[s] != BC_BOUNCEBACK && g.bc[s] != BC_FREESLIP) continue;
-        const double w = s == 0 ? -0.5 : (s == 1 ? g.nx - 0.5 : (s == 2 ? -0.5 : g.ny - 0.5));
-        if (s < 2) collision_force(B, B.radius, B.xc[0] - (2.0 * w - B.xc[0]), 0.0, Fc);
-        else collision_force(B, B.radius, 0.0, B.xc[1] - (2.0 * w - B.xc[1]), Fc);
+  // Eq. 39 of body i from partner o: bodies 0 .. nb - 1, then the four sides
+  auto partner = [&](const BodyDev& Bi, int i, int o, double* F) {
+    if (o < nb) {
+      if (o == i || bodies[o].kind != IBM_BODY_FREE) return;
+      collision_force(Bi, bodies[o].radius, Bi.xc[0] - bodies[o].xc[0], Bi.xc[1] - bodies[o].xc[1], F);
+      return;
+    }
+    const int s = o - nb;
+    if (g.bc[s] != BC_BOUNCEBACK && g.bc[s] != BC_FREESLIP) return;
+    const double w = s == 0 ? -0.5 : (s == 1 ? g.nx - 0.5 : (s == 2 ? -0.5 : g.ny - 0.5));
+    if (s < 2) collision_force(Bi, Bi.radius, Bi.xc[0] - (2.0 * w - Bi.xc[0]), 0.0, F);
+    else collision_force(Bi, Bi.radius, 0.0, Bi.xc[1] - (2.0 * w - Bi.xc[1]), F);
+  };
+  if (nb <= kPairBodies) {
+    // each partner's force by a thread of its own (a distance is an FP64
+    // square root, some 1,500 clocks), added up in the same order
+    __shared__ double pair[kPairBodies * (kPairBodies + 4)][2];
+    const int np = nb + 4;
+#pragma unroll 1
+    for (int k = b; k < nb * np; k += blockDim.x) {
+      const int i = k / np;
+      double F[2] = {0.0, 0.0};
+      if (bodies[i].kind == IBM_BODY_FREE) partner(bodies[i], i, k - i * np, F);
+      pair[k][0] = F[0];
+      pair[k][1] = F[1];
+    }
+    __syncthreads();
+    if (b < nb) {
+      B = bodies[b];
+#pragma unroll 1
+      for (int o = 0; o < np; ++o) {
+        Fc[0] += pair[b * np + o][0];
+        Fc[1] += pair[b * np + o][1];
       }
     }
+  } else if (b < nb) {
+    B = bodies[b];
+    if (B.kind == IBM_BODY_FREE)
+      for (int o = 0; o < nb + 4; ++o) partner(B, b, o, Fc);
   }
   __syncthreads();   // every body read the old positions before any update
   if (b >= nb) return;

@@ -175,7 +175,7 @@ namespace ibm {
 // Number of CUDA kernels one time step launches (matches enqueue_step; timed:
 // with the collide+stream launch bracketed).
 inline int kernels_per_step(const Ctx& h, bool timed = false) {
-  if (h.sl_on && !timed) return 2;                 // the correction, everything else
+  if (h.sl_on && !timed) return h.any_moving ? 3 : 2;   // correction, everything else, motion and rebuild
   int k = 1;                                       // collide + stream
   if (has_nee(h.geom)) k += 1;                     // extrapolation columns
   if (h.nm > 0) {
@@ -183,7 +183,7 @@ inline int kernels_per_step(const Ctx& h, bool timed = false) {
     // band collide+stream
     k += h.ib_phases == 1 ? h.desc.n_corr + 4
          : (h.ib_phases == 2 && h.ib_jc_cluster >= 2 ? (h.desc.n_corr > 1 ? 4 : 3) : 2);
-    if (h.nb > 0 && h.any_moving) k += 2 + 6;      // body update, marker move, band rebuild
+    if (h.nb > 0 && h.any_moving) k += h.sl_on ? 1 : 2 + 6;   // body update, marker move, band rebuild
   }
   return k;
 }
@@ -339,6 +339,11 @@ cudaError_t launch_slice_build(const Ctx& h, int* stat, cudaStream_t s);
 // Dynamic shared memory of the slice kernel (0: it does not fit).
 size_t slice_smem(const Ctx& h);
 int slice_max_corr();
+// Moving bodies: one slice holds every marker; sets its capacities (false: the
+// lattice keeps the general path).  launch_rebuild brings its lists and the
+// band up to the bodies' pose, after moving the bodies by a step if asked.
+bool slice_moving_fits(Ctx& h);
+cudaError_t launch_rebuild(const Ctx& h, bool move, cudaStream_t s);
 void launch_slice_loop(const Ctx& h, int parity, bool macro, cudaStream_t s);
 // The whole step in two launches on s (the correction, and one kernel for
 // everything else behind it); false: not on slices, or a grid too large.

@@ -226,21 +226,53 @@ __device__ __forceinline__ void copy16_async(void* dst, const void* src) {
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// The loop of ib_step_body by one CTA, for a moving boundary whose band did
+// not fit the slice's lists this step, with its results where k_slice_stream
+// looks for them.
 template <int P, int PAR>
+__device__ __noinline__ void slice_fallback(const IbArgs<P>& a, const SliceArgs<typename Prec<P>::R>& sl) {
+  typedef typename Prec<P>::R R;
+  ib_step_body<P, PAR, kSliceThreads>(a, 0, 1);
+  __syncthreads();
+  const int nband = min(a.ctr[CTR_NBAND], a.bcap), N = a.N;
+  for (int b = threadIdx.x; b < nband; b += kSliceThreads) {
+    R pxx = R(0), pxy = R(0), pyy = R(0);
+    for (int j = 0; j < a.bcnt[b]; ++j) {
+      const Ent<R> q = a.ent[(long long)b * kBandCap + j];
+      pxx += q.w * a.Cm[3 * q.m];
+      pxy += q.w * a.Cm[3 * q.m + 1];
+      pyy += q.w * a.Cm[3 * q.m + 2];
+    }
+    R* o = a.bq + 8 * (long long)b;
+    o[3] = pxx;
+    o[4] = pxy;
+    o[5] = pyy;
+  }
+  if (PAR == 1)
+    for (int k = threadIdx.x; k < 2 * a.M; k += kSliceThreads)
+      a.Ah[(long long)(N + 1) * 2 * a.M + k] = a.Ah[(long long)N * 2 * a.M + k];
+  for (int n = threadIdx.x; n <= N; n += kSliceThreads)
+    sl.rpart[(size_t)PAR * sl.count * (kSliceMaxCorr + 2) + n] = a.resid[n];
+}
+
+// MOVING: one slice holds every marker, its lists rebuilt by k_rebuild after
+// every step.
+template <int P, int PAR, bool MOVING>
 __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, SliceArgs<typename Prec<P>::R> sl) {
   typedef typename Prec<P>::R R;
   typedef typename Vec2<R>::T V;
   constexpr int NT = kSliceThreads;
   constexpr bool F64 = sizeof(R) == 8;
+  constexpr bool PAIRS = F64 && !MOVING;                     // few nodes: (node, n) pairs fill the warps
   constexpr int U = F64 ? 2 : 4;                             // nodes gathered at once per thread
-  constexpr int kLevels = 11;                                // iterates of the history read at once
+  constexpr int kLevels = F64 ? 6 : 11;                                // iterates of the history read at once
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = a.N, LM = sl.lmax, XM = sl.xmax, X1M = sl.x1max, EM = sl.emax;
   const int SM = (sl.S + 3) & ~3;
   V* hist = reinterpret_cast<V*>(smem_raw);                  // [N + 1][LM] A^n
   V* djs = hist + (size_t)(N + 1) * LM;                      // [N + 1][SM] dj^n of the owned markers
-  V* jn = djs + (size_t)(N + 1) * SM;                      // FP64: [N + 1][X1M] spread A^n
-  R* nr = reinterpret_cast<R*>(jn + (F64 ? (size_t)(N + 1) * X1M : 0));   // [XM] rho, jx, jy
+  V* jn = djs + (size_t)(N + 1) * SM;                      // PAIRS: [N + 1][X1M] spread A^n
+  R* nr = reinterpret_cast<R*>(jn + (PAIRS ? (size_t)(N + 1) * X1M : 0));   // [XM] rho, jx, jy
   R* njx = nr + XM;
   R* njy = njx + XM;
   R* sxx = njy + XM;                                         // [X1M] sum_n j^n j^n
@@ -262,6 +294,10 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
   const int own = head[4], nloc = head[4 + N], d1 = head[5];
   const size_t sm = (size_t)s * kSliceMarkers;
   dependency_release();                                      // k_slice_stream starts beside this kernel
+  if (MOVING && head[3]) {
+    slice_fallback<P, PAR>(a, sl);
+    return;
+  }
 #pragma unroll 1
   for (int k = t; k <= N; k += NT) {
     depth[k] = head[4 + k];
@@ -451,7 +487,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
 
   // per node of a depth <= 1 marker: sum_n j^n j^n; per owned node the summed
   // momentum correction D^N
-  if (F64) {
+  if (PAIRS) {
     // (node, n) pairs fill the warps; the sums over n follow in order
 #pragma unroll 1
     for (int k = t; k < (N + 1) * nX1; k += NT) {
@@ -477,7 +513,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
     const R j0x = njx[k], j0y = njy[k];
     R axx = R(0), axy = R(0), ayy = R(0);
     R* o = a.bq + 8 * (long long)sbid[k < nown ? k : 0];
-    if (F64) {
+    if (PAIRS) {
 #pragma unroll 1
       for (int n = 0; n < N; ++n) {
         const V p = jn[(size_t)n * X1M + k];
@@ -787,6 +823,289 @@ __global__ void __launch_bounds__(kStepThreads, k1_min_blocks(P, PAR))
   if (k < sh.nblk) band_block<P, PAR, MACRO, MRT, kStepThreads, true>(a, k, sh.nblk);
 }
 
+// ------------------------------------------------------------------ moving bodies
+// After a step of a lattice with moving bodies, one CTA: the Newton-Euler
+// update (Eqs. 37-42), the rigid motion of the markers, and the band and the
+// lists of its single slice for the next step -- in one launch where the
+// general path takes nine, each waiting for the one before, and builds the
+// rows of G one marker to a thread (48 us of the 118 us of a step with two
+// disks of 63 markers).  Here a warp finds the few markers that a marker
+// couples with by their windows and forms their G_lm a lane each; weights are
+// formed per axis (8 instead of 32 cosines a marker: FP64 issues at two lanes a
+// clock).  Every number is formed by the expressions of the general path in the
+// same order.  A band that does not fit (more nodes or covering markers than
+// the lists hold, a periodic axis shorter than two windows) is built by the
+// general path's items in the same CTA and flagged in head[3].
+constexpr int kRebuildThreads = 1024;
+template <class R>
+struct RebuildArgs {
+  Geom g;
+  int M, nb, N, points, nseg_x, bcap, segcap, move;
+  int xcap, ecap;                  // nodes and covering markers that the lists hold
+  BodyDev* bodies;
+  const int* mbody;
+  const double *dX, *dY, *ds;
+  double *X, *Y;
+  R *Ux, *Uy;
+  int *node2band, *bnode, *segflag, *seglist, *ctr;
+  // the general path's arrays
+  R* W;
+  int *node_of, *claim, *band_of, *bcnt, *gcnt;
+  Ent<R> *ent, *G;
+};
+
+// Shared memory of k_rebuild: weights of the stencil slots and their products
+// with ds, the axis weights, node table, covering lists.
+template <class R>
+struct RebuildShared {
+  double wx[2][4][kSliceMarkers];          // axis weights
+  double cs[kSliceMarkers], sn[kSliceMarkers];   // of the bodies
+  R w[kStencil][kSliceMarkers], wds[kStencil][kSliceMarkers];
+  int key[kSliceNodeHash];
+  unsigned short val[kSliceNodeHash];
+  unsigned short at[kStencil][kSliceMarkers];    // local node, 0xffff: outside
+  int node[kSliceX1], cnt[kSliceX1];
+  unsigned short list[kSliceEnt][kSliceX1];      // marker * 16 + slot
+  int bx[kSliceMarkers], by[kSliceMarkers];
+  unsigned short cand[kSliceRow][kSliceMarkers]; // coupled markers, ascending
+  int rows[kSliceMarkers];
+  int nn, nseg, bad;
+};
+
+// Difference of two window origins on one axis, the shorter way round.
+__device__ __forceinline__ int window_step(int d, int n, bool periodic) {
+  if (periodic) {                                // bodies may be whole periods apart
+    d %= n;
+    if (d > n / 2) d -= n;
+    else if (d < -(n / 2)) d += n;
+  }
+  return d;
+}
+
+template <class R>
+__global__ void __launch_bounds__(kRebuildThreads) k_rebuild(RebuildArgs<R> a, SliceArgs<R> sl) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  RebuildShared<R>& sh = *reinterpret_cast<RebuildShared<R>*>(smem_raw);
+  constexpr int NT = kRebuildThreads;
+  const Geom& g = a.g;
+  const int t = threadIdx.x, M = a.M;
+  const bool px = g.bc[0] == BC_PERIODIC, py = g.bc[2] == BC_PERIODIC;
+  // (slot, marker) pairs: marker ml, slots mq, mq + mstep, ..
+  const int mshift = M <= 64 ? 6 : (M <= 128 ? 7 : 8), mstep = NT >> mshift;
+  const int ml = t & ((1 << mshift) - 1), mq = ml < M ? t >> mshift : 64;
+  // the old band leaves the maps; the table is cleared
+  const int nold = min(a.ctr[CTR_NBAND], a.bcap);
+  for (int b = t; b < nold; b += NT) band_clear_item(g, a.bnode, a.node2band, a.segflag, a.nseg_x, b);
+  for (int k = t; k < kSliceNodeHash; k += NT) sh.key[k] = -1;
+  for (int k = t; k < a.xcap; k += NT) sh.cnt[k] = 0;
+  if (t == 0) { sh.nn = 0; sh.nseg = 0; sh.bad = (px && g.nx < 8) || (py && g.ny < 8); }
+  if (a.move) {
+    body_update_cta(g, a.bodies, a.nb);
+    if (t < a.nb) sincos(a.bodies[t].theta - a.bodies[t].theta0, &sh.sn[t], &sh.cs[t]);
+  }
+  __syncthreads();
+  if (t == 0) { a.ctr[CTR_NBAND] = 0; a.ctr[CTR_NSEG] = 0; }
+  if (t < M) {
+    double X, Y;
+    const int mb = a.mbody[t];
+    const BodyDev& B = a.bodies[mb];
+    if (a.move && B.kind != IBM_BODY_FIXED) {                // marker_move_item
+      const double cs = sh.cs[mb], sn = sh.sn[mb];
+      X = B.xc[0] + cs * a.dX[t] - sn * a.dY[t];
+      Y = B.xc[1] + sn * a.dX[t] + cs * a.dY[t];
+      a.X[t] = X;
+      a.Y[t] = Y;
+      a.Ux[t] = (R)(B.u[0] - B.omega * (Y - B.xc[1]));
+      a.Uy[t] = (R)(B.u[1] + B.omega * (X - B.xc[0]));
+    } else {
+      X = a.X[t];
+      Y = a.Y[t];
+    }
+    const int bx = (int)floor(X) - 1, by = (int)floor(Y) - 1;
+    sh.bx[t] = bx;
+    sh.by[t] = by;
+    sh.wx[0][0][t] = X;
+    sh.wx[1][0][t] = Y;
+  }
+  __syncthreads();
+  // axis weights; each pass keeps the position in slot 0 until it is replaced
+  double aw[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int k = t + q * NT;
+    if (k < 8 * M) {
+      const int l = k >> 3, ax = (k >> 2) & 1, i = k & 3;
+      aw[q] = delta_w(a.points, sh.wx[ax][0][l] - (double)((ax ? sh.by[l] : sh.bx[l]) + i));
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int k = t + q * NT;
+    if (k < 8 * M) sh.wx[(k >> 2) & 1][k & 3][k >> 3] = aw[q];
+  }
+  __syncthreads();
+  // stencil weights, nodes
+#pragma unroll 1
+  for (int q = mq; q < kStencil; q += mstep) {
+    const int l = ml;
+    const int x = wrap_axis(sh.bx[l] + (q & 3), g.nx, px), y = wrap_axis(sh.by[l] + (q >> 2), g.ny, py);
+    double w = 0.0;
+    unsigned short at = 0xffff;
+    if (x >= 0 && y >= 0) {
+      w = sh.wx[0][q & 3][l] * sh.wx[1][q >> 2][l];
+      bool fresh;
+      const int slot = table_insert(sh.key, sh.val, kSliceNodeHash, y * g.nx + x, &sh.nn, a.xcap, &fresh);
+      if (slot < 0) sh.bad = 1;
+      else {
+        at = (unsigned short)slot;                           // the value is complete after the barrier
+        if (fresh) sh.node[sh.val[slot]] = y * g.nx + x;
+      }
+    }
+    const R wr = (R)w;
+    sh.w[q][l] = wr;
+    sh.wds[q][l] = (R)((double)wr * a.ds[l]);
+    sh.at[q][l] = at;
+  }
+  __syncthreads();
+  const int nn = min(sh.nn, a.xcap);
+  if (!sh.bad) {
+    // covering lists: entries in any order, then by marker
+#pragma unroll 1
+    for (int q = mq; q < kStencil; q += mstep) {
+      const int l = ml;
+      if (sh.at[q][l] == 0xffff) continue;
+      const int n = sh.val[sh.at[q][l]];
+      sh.at[q][l] = (unsigned short)n;
+      const int pos = atomicAdd(&sh.cnt[n], 1);
+      if (pos < a.ecap) sh.list[pos][n] = (unsigned short)(l * kStencil + q);
+      else sh.bad = 1;
+    }
+  }
+  __syncthreads();
+  if (!sh.bad) {
+    for (int k = t; k < nn; k += NT) {
+      const int c = sh.cnt[k], n = sh.node[k];
+      for (int i = 1; i < c; ++i) {
+        const unsigned short v = sh.list[i][k];
+        int j = i - 1;
+        while (j >= 0 && sh.list[j][k] > v) { sh.list[j + 1][k] = sh.list[j][k]; --j; }
+        sh.list[j + 1][k] = v;
+      }
+      sl.nid[k] = n;
+      sl.bid[k] = k;
+      sl.en[k] = c;
+      for (int j = 0; j < a.ecap; ++j) {
+        const unsigned short v = j < c ? sh.list[j][k] : 0;
+        sl.ew[(size_t)j * kSliceX1 + k] = j < c ? sh.wds[v % kStencil][v / kStencil] : R(0);
+        sl.ei[(size_t)j * kSliceX1 + k] = (unsigned short)(v / kStencil);
+      }
+      a.bnode[k] = n;
+      a.node2band[n] = k;
+      const int y = n / g.nx, seg = y * a.nseg_x + (n - y * g.nx) / kSegW;
+      if (atomicCAS(&a.segflag[seg], 0, 1) == 0) {
+        const int at = atomicAdd(&sh.nseg, 1);
+        if (at < a.segcap) a.seglist[at] = seg;
+        else atomicOr(&a.ctr[CTR_ERR], ERR_SEG_CAP);
+      }
+    }
+    // coupled markers: those whose windows share a node inside the domain
+    const int warp = t >> 5, lane = t & 31;
+#pragma unroll 1
+    for (int l = warp; l < M; l += NT / 32) {
+      const int bx = sh.bx[l], by = sh.by[l];
+      int nc = 0;
+#pragma unroll 1
+      for (int m0 = 0; m0 < M; m0 += 32) {
+        const int m = m0 + lane;
+        bool near = false;
+        if (m < M) {
+          const int dx = window_step(sh.bx[m] - bx, g.nx, px), dy = window_step(sh.by[m] - by, g.ny, py);
+          int x0 = bx + max(dx, 0), x1 = bx + min(dx, 0) + 3, y0 = by + max(dy, 0), y1 = by + min(dy, 0) + 3;
+          if (!px) { x0 = max(x0, 0); x1 = min(x1, g.nx - 1); }
+          if (!py) { y0 = max(y0, 0); y1 = min(y1, g.ny - 1); }
+          near = x0 <= x1 && y0 <= y1;
+        }
+        const unsigned int hit = __ballot_sync(0xffffffffu, near);
+        const int pos = nc + __popc(hit & ((1u << lane) - 1u));
+        if (near && pos < kSliceRow) sh.cand[pos][l] = (unsigned short)m;
+        nc += __popc(hit);
+      }
+      if (lane == 0) {
+        sh.rows[l] = min(nc, kSliceRow);
+        if (nc > kSliceRow) sh.bad = 1;
+      }
+    }
+    __syncthreads();
+    // their G_lm, a pair per thread, summed over the shared nodes in slot
+    // order; rows padded to kRowHead with the marker itself at weight zero
+#pragma unroll 1
+    for (int q = mq; q < kSliceRow; q += mstep) {
+      const int l = ml, c = sh.rows[l];
+      if (q >= max(c, kRowHead)) break;
+      int m = l;
+      R acc = R(0);
+      if (q < c) {
+        m = sh.cand[q][l];
+        const int dx = window_step(sh.bx[m] - sh.bx[l], g.nx, px), dy = window_step(sh.by[m] - sh.by[l], g.ny, py);
+        bool has = false;
+#pragma unroll 1
+        for (int j = max(0, dy); j < min(4, 4 + dy); ++j)
+#pragma unroll 1
+          for (int i = max(0, dx); i < min(4, 4 + dx); ++i) {
+            if (sh.at[4 * j + i][l] == 0xffff) continue;
+            const R v = sh.w[4 * j + i][l] * sh.wds[4 * (j - dy) + i - dx][m];
+            if (has) acc += v;
+            else acc = v;
+            has = true;
+          }
+      }
+      sl.rw[(size_t)q * kSliceMarkers + l] = acc;
+      sl.ri[(size_t)q * kSliceMarkers + l] = (unsigned short)m;
+    }
+    if (t < M) sl.rn[t] = sh.rows[t];
+#pragma unroll 1
+    for (int q = mq; q < kStencil; q += mstep) sl.w[(size_t)q * kSliceMarkers + ml] = sh.w[q][ml];
+#pragma unroll 1
+    for (int q = mq; q < kStencil / 2; q += mstep) {
+      const unsigned int lo = sh.at[2 * q][ml], hi = sh.at[2 * q + 1][ml];
+      sl.wi[(size_t)q * kSliceMarkers + ml] = (lo == 0xffff ? 0u : lo) | ((hi == 0xffff ? 0u : hi) << 16);
+    }
+    if (t < M) sl.mid[t] = t;
+    for (int k = t; k < kSliceHead; k += NT) sl.head[k] = k < 3 ? nn : (k == 3 ? 0 : M);
+  }
+  __syncthreads();
+  if (!sh.bad) {
+    if (t == 0) { a.ctr[CTR_NBAND] = nn; a.ctr[CTR_NSEG] = min(sh.nseg, a.segcap); }
+    return;
+  }
+  // the general path, by this CTA (what the list pass above has entered in the
+  // maps leaves them first)
+  for (int k = t; k < nn; k += NT) {
+    const int n = sh.node[k], y = n / g.nx;
+    a.node2band[n] = -1;
+    a.segflag[y * a.nseg_x + (n - y * g.nx) / kSegW] = 0;
+  }
+  if (t == 0) sl.head[3] = 1;
+  __syncthreads();
+  const int T = M * kStencil;
+  for (int k = t; k < T; k += NT)
+    band_claim_item<R>(g, a.X, a.Y, a.W, a.node_of, a.node2band, a.claim, a.points, k);
+  __syncthreads();
+  for (int k = t; k < T; k += NT)
+    band_alloc_item(a.node_of, a.claim, a.node2band, a.bnode, a.bcnt, a.ctr, a.bcap, k);
+  __syncthreads();
+  for (int k = t; k < T; k += NT)
+    band_fill_item<R>(a.node_of, a.W, a.ds, a.node2band, a.band_of, a.bcnt, a.ent, a.ctr, k);
+  __syncthreads();
+  const int nnew = min(a.ctr[CTR_NBAND], a.bcap);
+  for (int b = t; b < nnew; b += NT) band_sort_item<R>(a.bcnt, a.ent, b);
+  for (int b = t; b < nnew; b += NT)
+    band_segment_item(g, a.bnode, a.segflag, a.seglist, a.ctr, a.nseg_x, a.segcap, b);
+  __syncthreads();
+  for (int l = t; l < M; l += NT) build_g_item<R>(a.band_of, a.W, a.bcnt, a.ent, a.G, a.gcnt, a.ctr, l);
+}
+
 // ------------------------------------------------------------------ launchers
 template <class R>
 static SliceArgs<R> slice_args(const Ctx& h) {
@@ -799,6 +1118,76 @@ static SliceArgs<R> slice_args(const Ctx& h) {
   s.emax = h.sl_emax;
   slice_bytes<R>(h.sl_count, (unsigned char*)h.sl_mem, &s);
   return s;
+}
+
+template <class R>
+static cudaError_t rebuild_t(const Ctx& h, bool move, cudaStream_t s) {
+  RebuildArgs<R> a{};
+  a.g = h.geom;
+  a.M = h.nm;
+  a.nb = h.nb;
+  a.N = h.desc.n_corr;
+  a.points = h.desc.delta_points;
+  a.nseg_x = h.nseg_x;
+  a.bcap = h.bcap;
+  a.segcap = h.segcap;
+  a.move = move ? 1 : 0;
+  a.xcap = h.sl_xmax;
+  a.ecap = h.sl_emax;
+  a.bodies = h.dbodies;
+  a.mbody = h.dmbody;
+  a.dX = h.ddX;
+  a.dY = h.ddY;
+  a.ds = h.dds;
+  a.X = h.dX;
+  a.Y = h.dY;
+  a.Ux = (R*)h.dUx;
+  a.Uy = (R*)h.dUy;
+  a.node2band = h.dnode2band;
+  a.bnode = h.dbnode;
+  a.segflag = h.dsegflag;
+  a.seglist = h.dseglist;
+  a.ctr = h.dctr;
+  a.W = (R*)h.dW;
+  a.node_of = h.dnode_of;
+  a.claim = h.dclaim;
+  a.band_of = h.dband_of;
+  a.bcnt = h.dbcnt;
+  a.gcnt = h.dgcnt;
+  a.ent = (Ent<R>*)h.dent;
+  a.G = (Ent<R>*)h.dG;
+  k_rebuild<R><<<1, kRebuildThreads, sizeof(RebuildShared<R>), s>>>(a, slice_args<R>(h));
+  return cudaPeekAtLastError();
+}
+
+cudaError_t launch_rebuild(const Ctx& h, bool move, cudaStream_t s) {
+  return h.r_bytes == 8 ? rebuild_t<double>(h, move, s) : rebuild_t<float>(h, move, s);
+}
+
+template <class R>
+static bool moving_fits_t(Ctx& h) {
+  h.sl_count = 1;
+  h.sl_S = h.nm;
+  h.sl_lmax = (h.nm + 31) / 32 * 32;
+  // a marker one lattice unit or less from the one before adds at most seven
+  // nodes to its window's sixteen
+  h.sl_xmax = h.sl_x1max = std::min(kSliceX1, (7 * h.nm + 32 + 31) / 32 * 32);
+  h.sl_nseg = std::min(h.segcap, std::max(64, h.nm));
+  if (cudaFuncSetAttribute(k_rebuild<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RebuildShared<R>)) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  for (int e : {12, 10, 8}) {
+    h.sl_emax = e;
+    if (slice_smem(h) > 0) return true;
+  }
+  return false;
+}
+
+bool slice_moving_fits(Ctx& h) {
+  if (h.nm > kSliceMarkers || h.nb > kRebuildThreads) return false;
+  return h.r_bytes == 8 ? moving_fits_t<double>(h) : moving_fits_t<float>(h);
 }
 
 int slice_max_corr() { return kSliceMaxCorr; }
@@ -835,7 +1224,7 @@ constexpr int kStepCarveout = 44;
 template <int P>
 static size_t slice_smem_t(const Ctx& h) {
   const size_t need = slice_smem_bytes<typename Prec<P>::R>(h.sl_xmax, h.sl_x1max, h.sl_lmax, h.sl_emax, h.sl_S,
-                                                            h.desc.n_corr);
+                                                            h.desc.n_corr, !h.any_moving);
   constexpr size_t kMax = 200 * 1024;
   if (need > kMax) return 0;
   bool ok = true;
@@ -843,8 +1232,13 @@ static size_t slice_smem_t(const Ctx& h) {
     if (slice) ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, kStepCarveout) == cudaSuccess;
   };
-  set(k_ib_slice<P, 0>, true);
-  set(k_ib_slice<P, 1>, true);
+  if (h.any_moving) {
+    set(k_ib_slice<P, 0, true>, true);
+    set(k_ib_slice<P, 1, true>, true);
+  } else {
+    set(k_ib_slice<P, 0, false>, true);
+    set(k_ib_slice<P, 1, false>, true);
+  }
   if (h.desc.collision == IBM_COLL_MRT) {
     set(k_slice_stream<P, 0, false, true>, false);
     set(k_slice_stream<P, 0, true, true>, false);
@@ -876,10 +1270,16 @@ template <int P>
 static void launch_slices(const Ctx& h, int parity, cudaStream_t s, const IbArgs<P>& a,
                           const SliceArgs<typename Prec<P>::R>& sl) {
   typedef typename Prec<P>::R R;
-  const size_t smem = slice_smem_bytes<R>(sl.xmax, sl.x1max, sl.lmax, sl.emax, sl.S, a.N);
+  const size_t smem = slice_smem_bytes<R>(sl.xmax, sl.x1max, sl.lmax, sl.emax, sl.S, a.N, !h.any_moving);
   const dim3 grid(sl.count), block(kSliceThreads);
-  if (parity == 0) launch_prio_smem(k_ib_slice<P, 0>, grid, block, smem, s, h.ib_prio, a, sl);
-  else launch_prio_smem(k_ib_slice<P, 1>, grid, block, smem, s, h.ib_prio, a, sl);
+  auto go = [&](auto kern) { launch_prio_smem(kern, grid, block, smem, s, h.ib_prio, a, sl); };
+  if (h.any_moving) {
+    if (parity == 0) go(k_ib_slice<P, 0, true>);
+    else go(k_ib_slice<P, 1, true>);
+  } else {
+    if (parity == 0) go(k_ib_slice<P, 0, false>);
+    else go(k_ib_slice<P, 1, false>);
+  }
 }
 
 template <int P>

@@ -105,13 +105,14 @@ inline size_t slice_bytes(int count, unsigned char* base, SliceArgs<R>* s) {
 }
 
 // Dynamic shared memory of one slice CTA, in the order of its pieces: the A
-// history, the owned markers' dj^n, (FP64) j^n of the depth <= 1 markers'
+// history, the owned markers' dj^n, (FP64, pairs) j^n of the depth <= 1 markers'
 // nodes; rho, j of the nodes; sum_n j^n j^n; C; W / rho; rho* of the owned
 // markers; the covering lists' weights and counts, the band indices, the
 // lists' markers; the nodes of W / rho.
 template <class R>
-__host__ __device__ constexpr size_t slice_smem_bytes(int xmax, int x1max, int lmax, int emax, int S, int N) {
-  return 2 * sizeof(R) * ((size_t)(N + 1) * (lmax + ((S + 3) & ~3)) + (sizeof(R) == 8 ? (size_t)(N + 1) * x1max : 0)) +
+__host__ __device__ constexpr size_t slice_smem_bytes(int xmax, int x1max, int lmax, int emax, int S, int N,
+                                                       bool pairs) {
+  return 2 * sizeof(R) * ((size_t)(N + 1) * (lmax + ((S + 3) & ~3)) + (sizeof(R) == 8 && pairs ? (size_t)(N + 1) * x1max : 0)) +
          sizeof(R) * ((size_t)3 * xmax + (size_t)3 * x1max + (size_t)3 * lmax + ((S + 3) & ~3)) +
          (size_t)emax * x1max * (sizeof(R) + sizeof(short)) + (size_t)x1max * 2 * sizeof(int) +
          (size_t)kStencil * lmax * (sizeof(R) + sizeof(short));

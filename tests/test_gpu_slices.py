@@ -112,3 +112,62 @@ def test_slices_follow_added_bodies_and_marker_velocities():
         lat.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+MOVING = {
+    # two disks, one free disk near a wall, prescribed motion across the periodic edge
+    "pair": lambda: wl.settling_pair(nx=64, ny=130, diameter=10.0, density_ratio=1.2, gravity=2e-4),
+    "wall": lambda: wl.Case("wall", 41, 90, 0.8, bc=(wl.BOUNCEBACK,) * 4,
+                            bodies=[wl.disk(9.2, 70.0, 14.0, 1.3, 3e-4)]),
+    "edge": lambda: _prescribed((1.3, 60.2)),
+    # touching disks: nodes covered by both rings
+    "touch": lambda: wl.Case("touch", 72, 72, 0.8, bc=(wl.BOUNCEBACK,) * 4,
+                             bodies=[wl.disk(28.0, 36.0, 16.0, 1.2, 1e-4), wl.disk(44.6, 36.0, 16.0, 1.2, 1e-4)]),
+    # a fixed ring around a free disk; 256 markers; half a unit apart (lists too long: the general path)
+    "mixed": lambda: _mixed(),
+    "most": lambda: _free_ring(40.0, 256),
+    "dense": lambda: _free_ring(16.0, 200),
+}
+
+
+def _prescribed(at):
+    xy, ds = wl.ring(at[0], at[1], 9.0)
+    b = wl.Body(xy, ds, wl.BODY_PRESCRIBED, xc=at, u=(0.08, -0.05), omega=0.01, radius=9.0)
+    return wl.Case("prescribed", 64, 61, 0.8, bodies=[b])
+
+
+def _mixed():
+    c = _rings(80, (30.0,))
+    c.bodies.append(wl.disk(40.0, 41.0, 12.0, 1.2, 1e-4))
+    return c
+
+
+def _free_ring(radius, count):
+    b = wl.disk(60.2, 59.7, 2 * radius, 1.2, 1e-4)
+    xy, ds = wl.ring(60.2, 59.7, radius, count=count)
+    b.xy, b.ds = xy, ds
+    return wl.Case("free", 121, 120, 0.8, bc=(wl.BOUNCEBACK,) * 4, bodies=[b])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("name", sorted(MOVING))
+def test_moving_bodies_on_a_rebuilt_slice_are_bitwise_the_phase_kernels(name, prec):
+    case = MOVING[name]()
+    out = []
+    for phases in (0, 1):
+        lat = gpu_lattice(case, prec)
+        if phases:
+            ibm.ibm_set_option(lat.h, ibm.IBM_OPT_IB_PHASES, phases)
+        lat.step(19)
+        lat.step(1, ibm.STEP_NO_GRAPH)
+        band = lat.sizes()
+        # a pose written between steps, and a switch of the launch form on the way
+        lat.write(ibm.FIELD_BODY_STATE, lat.read(ibm.FIELD_BODY_STATE))
+        lat.step(3)
+        if not phases:
+            ibm.ibm_set_option(lat.h, ibm.IBM_OPT_IB_PHASES, 1)
+        lat.step(2)
+        out.append((lat.f, lat.resid, lat.bodies, lat.markers, np.array(band), *lat.moments()))
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
