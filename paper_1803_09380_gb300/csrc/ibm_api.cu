@@ -160,10 +160,13 @@ ibm_status check_device_flags(Ctx* h) {
   return IBM_OK;
 }
 
+// One wait: the copy of the flags is ordered behind the stream's work.
 ibm_status sync_stream(Ctx* h) {
-  IBM_CK(h, cudaStreamSynchronize(h->stream));
+  if (!h->dctr) IBM_CK(h, cudaStreamSynchronize(h->stream));
+  const ibm_status st = check_device_flags(h);
+  if (st != IBM_OK) return st;
   IBM_CK(h, cudaGetLastError());
-  return check_device_flags(h);
+  return IBM_OK;
 }
 
 ibm_status ensure_io(Ctx* h, size_t doubles) {
@@ -272,9 +275,12 @@ void choose_ib_grid(Ctx& c) {
 // Markers that one slice of the barrier-free correction owns when the caller
 // has not set a CTA count: an even share for every SM, between a smallest
 // slice (below it the neighbourhood outweighs what it saves) and the largest
-// that leaves room for the neighbourhood of ten iterations.
+// that leaves room for the neighbourhood of ten iterations.  (us a step, FP64
+// 64^2 with 220 markers: slices of 16, 8, 4, 2: 39.0, 36.7, 35.6, 35.4; FP32
+// 300^2 with 1029 markers: 32, 16, 8, 7: 12.6, 11.8, 11.9, 12.3; 1024^2 with
+// 3513 markers: 64, 32, 24: 19.2, 17.5, 17.7.)
 int slice_size(const Ctx& c) {
-  const int lo = c.r_bytes == 8 ? 8 : 16;
+  const int lo = c.r_bytes == 8 ? 4 : 8;
   return std::max(lo, std::min(128, (c.nm + c.ib_grid_max - 1) / c.ib_grid_max));
 }
 
@@ -362,7 +368,7 @@ ibm_status upload_markers(Ctx* h) {
   Ctx& c = *h;
   const int M = c.nm;
   // release the previous marker-sized buffers
-  void* olds[] = {c.dX, c.dY, c.dds, c.ddX, c.ddY, c.dmbody, c.dUx, c.dUy, c.dW, c.dnode_of,
+  void* olds[] = {c.dX, c.dY, c.dds, c.ddX, c.ddY, c.dmbody, c.dUx, c.dW, c.dnode_of,
                   c.dband_of, c.dclaim, c.dbnode, c.dbcnt, c.dent, c.dbq, c.dmq, c.dAh,
                   c.dCm, c.dG, c.dgcnt, c.dbodies, c.dfpart};
   IBM_CK(h, cudaStreamSynchronize(c.stream));
@@ -384,8 +390,8 @@ ibm_status upload_markers(Ctx* h) {
   IBM_ALLOC(h, c.ddX, double*, M);
   IBM_ALLOC(h, c.ddY, double*, M);
   IBM_ALLOC(h, c.dmbody, int*, M);
-  c.dUx = dev_alloc(c, R * M);
-  c.dUy = dev_alloc(c, R * M);
+  c.dUx = dev_alloc(c, R * 2 * (size_t)M);          // dUy follows: prescribed velocities go in one copy
+  c.dUy = c.dUx ? (char*)c.dUx + R * (size_t)M : nullptr;
   c.dW = dev_alloc(c, R * M * kStencil);
   IBM_ALLOC(h, c.dnode_of, int*, M * kStencil);
   IBM_ALLOC(h, c.dband_of, int*, M * kStencil);
@@ -858,15 +864,16 @@ ibm_status ibm_set_marker_velocities(ibm_handle h, const double* uv, int n) {
     if (!guard.ok) return fail(h, IBM_ERR_CUDA, "cannot select the CUDA device");
     Ctx& c = *h;
     const int R = c.r_bytes;
-    std::vector<char> ux((size_t)R * n), uy((size_t)R * n);
+    std::vector<char> u(2 * (size_t)R * n);
+    char *ux = u.data(), *uy = ux + (size_t)R * n;
     for (int l = 0; l < n; ++l) {
       if (c.hbodies[c.hmbody[l]].kind != IBM_BODY_FIXED) continue;
       c.hUx[l] = uv[2 * l];
       c.hUy[l] = uv[2 * l + 1];
     }
     for (int l = 0; l < n; ++l) {
-      if (R == 8) { ((double*)ux.data())[l] = c.hUx[l]; ((double*)uy.data())[l] = c.hUy[l]; }
-      else { ((float*)ux.data())[l] = (float)c.hUx[l]; ((float*)uy.data())[l] = (float)c.hUy[l]; }
+      if (R == 8) { ((double*)ux)[l] = c.hUx[l]; ((double*)uy)[l] = c.hUy[l]; }
+      else { ((float*)ux)[l] = (float)c.hUx[l]; ((float*)uy)[l] = (float)c.hUy[l]; }
     }
     // Pageable sources are staged before cudaMemcpyAsync returns, so the
     // temporaries may go; the copies are ordered before the next step.
@@ -878,15 +885,14 @@ ibm_status ibm_set_marker_velocities(ibm_handle h, const double* uv, int n) {
         if (c.hbodies[c.hmbody[l]].kind != IBM_BODY_FIXED) { ++l; continue; }
         int e = l;
         while (e < n && c.hmbody[e] == c.hmbody[l]) ++e;
-        IBM_CK(h, cudaMemcpyAsync((char*)c.dUx + (size_t)R * l, ux.data() + (size_t)R * l, (size_t)R * (e - l),
+        IBM_CK(h, cudaMemcpyAsync((char*)c.dUx + (size_t)R * l, ux + (size_t)R * l, (size_t)R * (e - l),
                                   cudaMemcpyHostToDevice, c.stream));
-        IBM_CK(h, cudaMemcpyAsync((char*)c.dUy + (size_t)R * l, uy.data() + (size_t)R * l, (size_t)R * (e - l),
+        IBM_CK(h, cudaMemcpyAsync((char*)c.dUy + (size_t)R * l, uy + (size_t)R * l, (size_t)R * (e - l),
                                   cudaMemcpyHostToDevice, c.stream));
         l = e;
       }
     } else {
-      IBM_CK(h, cudaMemcpyAsync(c.dUx, ux.data(), (size_t)R * n, cudaMemcpyHostToDevice, c.stream));
-      IBM_CK(h, cudaMemcpyAsync(c.dUy, uy.data(), (size_t)R * n, cudaMemcpyHostToDevice, c.stream));
+      IBM_CK(h, cudaMemcpyAsync(c.dUx, ux, 2 * (size_t)R * n, cudaMemcpyHostToDevice, c.stream));
     }
     return IBM_OK;
   } catch (...) {
