@@ -362,11 +362,14 @@ def run_ours(args, rank, world, local_rank, dist):
     if args.ib_threads:
         lat.set_ib_threads(args.ib_threads)
     stream = lat._stream
-    flags = ibm.STEP_TIME_KERNELS | ibm.STEP_NO_MACRO
+    flags = ibm.STEP_NO_MACRO
 
+    # warm-up: the asked steps, then twice a stretch that ends as the timed call
+    # does, so that every graph it replays exists (8-step blocks, single steps)
     lat.step(max(args.warmup, 3), flags)
+    for _ in range(2):
+        lat.step(16 + args.steps % 8, flags)
     lat.sync()
-    lat.kernel_times()
     l0, _ = lat.counters()
 
     def barrier():
@@ -387,9 +390,15 @@ def run_ours(args, rank, world, local_rank, dist):
     barrier()
     clocks = sampler.stop() if sampler else None
     ms = e0.elapsed_time(e1)
-    k1_ms, k1_n = lat.kernel_times()
     l1, _ = lat.counters()
     launches = l1 - l0
+    # the dominant kernel by itself: steps in the form that brackets the band-free
+    # collide+stream launch with events
+    timed = ibm.STEP_TIME_KERNELS | ibm.STEP_NO_MACRO
+    lat.step(8, timed)
+    lat.kernel_times()
+    lat.step(min(args.steps, 200), timed)
+    k1_ms, k1_n = lat.kernel_times()
     ms = max_over_ranks(ms, dist, "cuda")
     value = whole_job_mlups(N2, args.steps, world, ms)
 
@@ -435,9 +444,10 @@ def run_ours(args, rank, world, local_rank, dist):
                 "dtype": DTYPE[args.prec], "data": "synthetic",
                 "config": workload_config(args, case),
                 "correction_ctas": tuned[0] if tuned else (args.ib_ctas or "library default"),
-                "timed_path": "ibm_step with IBM_STEP_TIME_KERNELS | IBM_STEP_NO_MACRO: every step "
+                "timed_path": "ibm_step with IBM_STEP_NO_MACRO (graph replays): every step "
                               "corrects, collides and streams; rho and u are not written out on the "
-                              "last step of the call (the optional output fields)",
+                              "last step of the call (the optional output fields); the roofline's "
+                              "launches are timed in a run of their own (IBM_STEP_TIME_KERNELS)",
                 "roofline": roofline, "cpu_baseline": cpu,
                 "e2e": e2e, "gpu_launches": launches, "clocks": clocks, "serving": serving}
         print(json.dumps(line), flush=True)

@@ -188,8 +188,11 @@ ibm_status ibm_add_markers(ibm_handle h, const double *xy, const double *ds,
  * the post-stream state (Eqs. 22-28; residuals r^0..r^N recorded), body
  * force and torque (Eq. 29), the body update (Eqs. 37-42) and marker motion,
  * then the fused BGK collide + AA-pattern stream over every node.  Returns
- * once the steps are enqueued, except with corr_tol > 0: then it waits for
- * them and returns IBM_WARN_NOT_CONVERGED if any step since the last
+ * once the steps are enqueued; the first call after markers were added or an
+ * option was set also waits for the lists it builds on the stream (a stream
+ * that is being captured is left alone: such a call runs the persistent
+ * kernel).  With corr_tol > 0 it waits for the steps
+ * and returns IBM_WARN_NOT_CONVERGED if any step since the last
  * synchronising call ended with r^N > corr_tol (or the error of a failed
  * step).  IBM_ERR_INVALID after a failed ibm_add_markers (destroy the
  * lattice). */
@@ -256,10 +259,16 @@ ibm_status ibm_set_marker_velocities(ibm_handle h, const double *uv, int n);
 
 /* Tuning options for ibm_set_option. */
 enum {
-  IBM_OPT_IB_CTAS = 1,  /* CTAs of the correction kernel: 0 (default) = one CTA for up to 512
-                           markers, 3 per 4 SMs above that; n > 0 = min(n, SMs).  2..16 CTAs
-                           run as one thread-block cluster when the device can schedule it.
-                           Results do not depend on it. */
+  IBM_OPT_IB_CTAS = 1,  /* CTAs of the correction kernel; n > 0 = min(n, SMs).  Markers that keep
+                           their places are dealt to the CTAs in slices, each iterated with
+                           the neighbourhood it depends on, without a barrier (0, the default:
+                           a slice per SM, of 4 (FP64) or 8 to 128 markers); up to 256 markers of
+                           moving bodies run on one CTA.  Where the slices do not fit (too few
+                           CTAs for the markers, very dense markers, more than 60 iterations)
+                           a persistent kernel with a grid barrier runs instead: 0 = one CTA
+                           for up to 512 markers, 3 per 4 SMs above that; 2..16 CTAs run as
+                           one thread-block cluster when the device can schedule it.  Results
+                           do not depend on it. */
   IBM_OPT_IB_THREADS = 2, /* threads per correction-kernel CTA: 256 (default), 512 or 1024 */
   IBM_OPT_WATCHDOG_STEPS = 3, /* K > 0: after every K steps (at the next 8-step block boundary)
                            scan every stored population for NaN/Inf; a hit makes the next
@@ -270,7 +279,8 @@ enum {
                            barrier in microseconds, [100, 6e7] (default 2 s); a wait that runs
                            out makes the next synchronising call return IBM_ERR_TIMEOUT */
   IBM_OPT_IB_PHASES = 6,     /* how the correction loop of section 2.3 is launched.  0 (default):
-                           one persistent kernel with a grid barrier between phases.  1: a chain
+                           slices, or one persistent kernel with a grid barrier between
+                           phases (see IBM_OPT_IB_CTAS).  1: a chain
                            of short kernels, one per phase (band gather, interpolation, each
                            Jacobi iteration, final residual and history, second moments),
                            ordered by the stream; their CTAs leave the SMs as soon as their
@@ -283,8 +293,9 @@ enum {
   IBM_OPT_TEST_DROP_ARRIVAL = 5 /* testing the timeout path only: 1 makes the last CTA of the
                            correction kernel skip its arrival at the first grid barrier of each
                            step, so the other CTAs' waits run out (bounded by
-                           IBM_OPT_BARRIER_LIMIT_US).  Only grids that wait at the
-                           global-memory barrier (more than 16 CTAs) are affected.  The
+                           IBM_OPT_BARRIER_LIMIT_US); it selects the persistent kernel.  Only
+                           grids that wait at the global-memory barrier (more than 16 CTAs)
+                           are affected.  The
                            lattice's results are then wrong; destroy it afterwards. */
 };
 
@@ -302,8 +313,8 @@ ibm_status ibm_autotune_ib(ibm_handle h, const int *candidates, int n, int steps
                            double *best_us);
 
 /* Sets a tuning option of h (takes effect at the next step).  Concurrency
- * note: a correction kernel of more than 16 CTAs (the default for more than
- * 512 markers) waits at a grid barrier in global memory and needs all its
+ * note: a persistent correction kernel of more than 16 CTAs (see
+ * IBM_OPT_IB_CTAS) waits at a grid barrier in global memory and needs all its
  * CTAs resident at once; step at most two such lattices at once on one GPU
  * (the server below keeps a budget).  Grids of 2..16 CTAs run as one
  * thread-block cluster, which the hardware schedules as a whole. */
