@@ -350,6 +350,29 @@ __device__ __forceinline__ void even_vec(const Geom& g, const StepConsts<typenam
   }
 }
 
+// All but one element of an aligned vector at p, in as few stores as its
+// alignment allows: elements 1 .. from o[0 .., or elements 0 .. from o[1 ...
+template <class S, int VEC>
+__device__ __forceinline__ void store_upper(S* p, const S (&o)[VEC]) {
+  p[1] = o[0];
+  if (VEC == 4) {
+    SVec<S, 2> v;
+    v.v[0] = o[VEC - 3 > 0 ? VEC - 3 : 0];
+    v.v[1] = o[VEC - 2];
+    vstore<S, 2>(p + 2, v);
+  }
+}
+template <class S, int VEC>
+__device__ __forceinline__ void store_lower(S* p, const S (&o)[VEC]) {
+  if (VEC == 4) {
+    SVec<S, 2> v;
+    v.v[0] = o[1];
+    v.v[1] = o[VEC - 2];
+    vstore<S, 2>(p, v);
+  }
+  p[VEC - 2] = o[VEC - 1];
+}
+
 // Odd step for one warp span of 32 * VEC consecutive nodes of row y that
 // holds no boundary node (periodic wrap only across the row ends).  Each
 // lane owns nodes x0 .. x0+VEC-1.  Loads and stores are aligned vectors; the
@@ -426,8 +449,7 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
       const S from_left = shfl_up1<S>(o[VEC - 1]);
       if (!skip) {
         if (lo) {
-#pragma unroll
-          for (int k = 0; k < VEC - 1; ++k) row[x0 + 1 + k] = o[k];
+          store_upper<S, VEC>(row + x0, o);
         } else {
           SVec<S, VEC> v;
           v.v[0] = from_left;
@@ -441,8 +463,7 @@ __device__ __forceinline__ void odd_vec(const Geom& g, const StepConsts<typename
       const S from_right = shfl_down1<S>(o[0]);
       if (!skip) {
         if (hi) {
-#pragma unroll
-          for (int k = 1; k < VEC; ++k) row[x0 + k - 1] = o[k];
+          store_lower<S, VEC>(row + x0, o);
         } else {
           SVec<S, VEC> v;
 #pragma unroll

@@ -17,9 +17,9 @@
 // whatever the slices.
 //
 // Measured against the persistent kernel with its band collide (us per step,
-// whole steps): 300^2 FP32 with 1029 markers 68.1 -> 16.4, 1024^2 FP32 with
-// 3513 markers 72.3 -> 21.6, 4096^2 FP32 with 14052 markers beside
-// collide+stream 220.8 -> 202.4, 64^2 FP64 with 220 markers 204.1 -> 39.0.
+// whole steps): 300^2 FP32 with 1029 markers 68.1 -> 12.0, 1024^2 FP32 with
+// 3513 markers 72.3 -> 17.5, 4096^2 FP32 with 14052 markers beside
+// collide+stream 220.8 -> 197.0, 64^2 FP64 with 220 markers 204.1 -> 35.8.
 //
 // What bounds it: latency.  The persistent kernel paid thirteen grid
 // barriers, each followed by dependent loads from L2; here the only global
