@@ -988,7 +988,11 @@ __global__ void __launch_bounds__(kRebuildThreads) k_rebuild(RebuildArgs<R> a, S
     }
   }
   __syncthreads();
-  if (!sh.bad) {
+  // every thread's branch is settled before a warp below may find a row that is
+  // too long: the barriers inside are met by all of them or by none
+  const bool fits = !sh.bad;
+  __syncthreads();
+  if (fits) {
     for (int k = t; k < nn; k += NT) {
       const int c = sh.cnt[k], n = sh.node[k];
       for (int i = 1; i < c; ++i) {

@@ -171,3 +171,69 @@ def test_moving_bodies_on_a_rebuilt_slice_are_bitwise_the_phase_kernels(name, pr
         lat.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def _window_counts(xy):
+    """Most markers that cover a node, and most markers that one couples with
+    (4 x 4 windows from floor(X) - 1 on, away from the sides)."""
+    o = np.floor(xy).astype(int) - 1
+    near = np.abs(o[:, None, :] - o[None, :, :])
+    rows = int(np.max(np.sum(np.all(near <= 3, axis=2), axis=1)))
+    grid = np.zeros(o.max(axis=0) + 4, int)
+    for x, y in o:
+        grid[x:x + 4, y:y + 4] += 1
+    return int(grid.max()), rows
+
+
+def _plates(k):
+    """Three plates of k x k markers two units apart in relative motion.  A node
+    is covered by at most four markers of a plate; a marker couples with nine
+    of its own plate and, as the window origins fall, with 9, 12 or 16 of each
+    other: at most 41, more than the lists' 32 rows in some poses."""
+    g = 2.0 * np.arange(k) - (k - 1)
+    xy = np.stack(np.meshgrid(g, g), -1).reshape(-1, 2)
+    bodies = []
+    for at, u in (((32.4, 31.3), (0.0, 0.0)), ((30.45, 29.35), (0.13, 0.02)), ((34.35, 31.4), (-0.03, 0.11))):
+        bodies.append(wl.Body(xy + at, np.ones(k * k), wl.BODY_PRESCRIBED, xc=at, u=u, radius=float(k)))
+    return wl.Case("plates", 64, 64, 0.8, bodies=bodies)
+
+
+def _crossing(r, m):
+    """Four rings on their way to one point: apart, at most six markers cover a
+    node; where they cross, up to 24, more than the lists hold."""
+    bodies = []
+    for dx, dy in ((-1, 0), (1, 0), (0, -1), (0, 1)):
+        at = (32.3 + (r + 2.2) * dx, 32.7 + (r + 2.2) * dy)
+        xy, ds = wl.ring(at[0], at[1], r, count=m)
+        bodies.append(wl.Body(xy, ds, wl.BODY_PRESCRIBED, xc=at, u=(-0.1 * dx, -0.1 * dy), radius=r))
+    return wl.Case("crossing", 64, 64, 0.8, bodies=bodies)
+
+
+@pytest.mark.parametrize("prec,make,limit", [
+    ("fp32", lambda: _plates(7), (12, 32)), ("fp64", lambda: _plates(5), (12, 32)),
+    ("fp32", lambda: _crossing(6.4, 40), (12, 32)), ("fp64", lambda: _crossing(4.0, 25), (12, 32))])
+def test_moving_bodies_in_and_out_of_what_the_slice_holds(prec, make, limit):
+    """Poses whose covering lists or rows do not fit the slice's take the general
+    path inside the same three launches a step, and the next pose that fits
+    comes back: every step bitwise the phase kernels."""
+    fast, ref = gpu_lattice(make(), prec), gpu_lattice(make(), prec)
+    ibm.ibm_set_option(ref.h, ibm.IBM_OPT_IB_PHASES, 1)
+    fit = []
+    for k in range(28):
+        if k == 14:                      # the way back
+            for lat in (fast, ref):
+                s = lat.read(ibm.FIELD_BODY_STATE)
+                s[:, 2:5] *= -1.0
+                lat.write(ibm.FIELD_BODY_STATE, s)
+        cover, rows = _window_counts(fast.markers)
+        fit.append(cover <= limit[0] and rows <= limit[1])
+        l0 = fast.counters()[0]
+        fast.step(1)
+        ref.step(1)
+        assert fast.counters()[0] - l0 == 3
+        assert np.array_equal(fast.bodies, ref.bodies) and np.array_equal(fast.resid, ref.resid)
+    assert fit[0] and fit[-1] and not all(fit)
+    assert np.all(np.isfinite(ref.f)) and np.array_equal(fast.f, ref.f)
+    assert np.array_equal(fast.markers, ref.markers)
+    fast.close()
+    ref.close()
