@@ -189,9 +189,12 @@ ibm_status ibm_add_markers(ibm_handle h, const double *xy, const double *ds,
  * force and torque (Eq. 29), the body update (Eqs. 37-42) and marker motion,
  * then the fused BGK collide + AA-pattern stream over every node.  Returns
  * once the steps are enqueued; the first call after markers were added or an
- * option was set also waits for the lists it builds on the stream (a stream
- * that is being captured is left alone: such a call runs the persistent
- * kernel).  With corr_tol > 0 it waits for the steps
+ * option was set also waits for the lists it builds on the stream.  A caller
+ * may capture the stream (IBM_STEP_NO_GRAPH; corr_tol 0; an even number of
+ * steps, since the in-place streaming alternates two kinds): nothing is built
+ * then, and where that call is the lattice's first, its steps and all later
+ * ones run the persistent kernel until markers are added.
+ * With corr_tol > 0 the call waits for the steps
  * and returns IBM_WARN_NOT_CONVERGED if any step since the last
  * synchronising call ended with r^N > corr_tol (or the error of a failed
  * step).  IBM_ERR_INVALID after a failed ibm_add_markers (destroy the

@@ -347,9 +347,24 @@ void plan_slices(Ctx& c) {
   c.sl_count = 0;
 }
 
+// The caller is capturing the lattice's stream into a graph of its own.
+bool being_captured(Ctx& c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c.stream, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
 // Forgets the slices (the band, or an option that they depend on, changes);
-// the caller has synchronised the stream and drops the graphs.
-void drop_slices(Ctx& c) {
+// the caller has synchronised the stream and drops the graphs.  A captured
+// step replays with the lists of its form, and the other form does not keep
+// them up (moving bodies) or numbers the band otherwise: the form then stays
+// until the markers are uploaded anew, which frees what the graph points to.
+void drop_slices(Ctx& c, bool markers = false) {
+  if (c.form_fixed && !markers) return;
+  c.form_fixed = false;
   if (c.sl_on && c.any_moving) c.band_valid = false;   // its rebuild leaves out the general path's lists
   if (c.sl_mem) dev_free(c, c.sl_mem);
   c.sl_mem = nullptr;
@@ -377,7 +392,7 @@ ibm_status upload_markers(Ctx* h) {
   IBM_CK(h, cudaMemsetAsync(c.dsegflag, 0, sizeof(int) * (size_t)c.nseg_x * c.geom.ny, c.stream));
   IBM_CK(h, cudaMemsetAsync(c.dctr, 0, CTR_COUNT * sizeof(int), c.stream));
   IBM_CK(h, cudaStreamSynchronize(c.stream));
-  drop_slices(c);
+  drop_slices(c, true);
   dev_free(c, c.dseglist);
   c.dseglist = nullptr;
   for (void* p : olds) dev_free(c, p);
@@ -796,6 +811,8 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
         if (st != IBM_OK) return st;
       }
     }
+    // the captured form of an unplanned lattice is the persistent kernel's
+    if (c.nm > 0 && !c.sl_tried && being_captured(c)) c.sl_tried = c.form_fixed = true;
     if (c.nm > 0 && !c.sl_tried) plan_slices(c);
     const bool want_macro = !(flags & IBM_STEP_NO_MACRO);
     for (int k = 0; k < nsteps;) {

@@ -135,6 +135,7 @@ struct Ctx {
   // barrier-free correction (ibm_slice.cuh): the slices of the current band
   bool sl_tried = false;                     // planned for the current band and options
   bool sl_on = false;                        // steps run on the slices
+  bool form_fixed = false;                   // the caller captured a step: no change of form (drop_slices)
   int sl_count = 0, sl_S = 0;                // slices, markers owned by each
   int sl_xmax = 0, sl_x1max = 0;             // largest local node counts
   int sl_lmax = 0, sl_emax = 0;              // largest marker count and covering list
