@@ -192,8 +192,10 @@ ibm_status ibm_add_markers(ibm_handle h, const double *xy, const double *ds,
  * option was set also waits for the lists it builds on the stream.  A caller
  * may capture the stream (IBM_STEP_NO_GRAPH; corr_tol 0; an even number of
  * steps, since the in-place streaming alternates two kinds): nothing is built
- * then, and where that call is the lattice's first, its steps and all later
- * ones run the persistent kernel until markers are added.
+ * then.  Where that call is the lattice's first, its steps and all later ones
+ * run the persistent kernel, otherwise the slices if they run by then; either
+ * way that form (see IBM_OPT_IB_CTAS), with its lists, stays until markers are
+ * added or the lattice is destroyed, whatever options are set.
  * With corr_tol > 0 the call waits for the steps
  * and returns IBM_WARN_NOT_CONVERGED if any step since the last
  * synchronising call ended with r^N > corr_tol (or the error of a failed

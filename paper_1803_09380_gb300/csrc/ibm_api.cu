@@ -811,8 +811,8 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
         if (st != IBM_OK) return st;
       }
     }
-    // the captured form of an unplanned lattice is the persistent kernel's
-    if (c.nm > 0 && !c.sl_tried && being_captured(c)) c.sl_tried = c.form_fixed = true;
+    // a captured step fixes the form; that of an unplanned lattice is the persistent kernel
+    if (c.nm > 0 && being_captured(c)) c.sl_tried = c.form_fixed = true;
     if (c.nm > 0 && !c.sl_tried) plan_slices(c);
     const bool want_macro = !(flags & IBM_STEP_NO_MACRO);
     for (int k = 0; k < nsteps;) {

@@ -61,3 +61,48 @@ def test_replays_of_a_captured_first_call_mixed_with_plain_steps(name, prec):
     lat.step(1)
     _same(lat, case, prec, 19)
     lat.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_options_set_after_a_capture_keep_what_the_graph_holds(name, prec):
+    """The slices run before the capture: options and the autotuner leave their
+    lists (and the form) alone, and the memory is not handed out again."""
+    import torch
+    case = CASES[name]()
+    lat = gpu_lattice(case, prec)
+    lat.step(3)
+    lat.step(1)
+    per_step = lat.counters()[0]
+    replay = _capture(lat, 2)
+    per_step = (lat.counters()[0] - per_step) // 2
+    assert per_step == (3 if name == "pair" else 2)          # slices
+    for option, value in ((ibm.IBM_OPT_IB_CTAS, 2), (ibm.IBM_OPT_IB_THREADS, 512),
+                          (ibm.IBM_OPT_IB_PHASES, 1), (ibm.IBM_OPT_BARRIER_LIMIT_US, 3000000)):
+        ibm.ibm_set_option(lat.h, option, value)
+    with torch.cuda.stream(lat._stream):
+        junk = [torch.full((1 << k,), 255, dtype=torch.uint8, device="cuda") for k in range(12, 25) for _ in range(4)]
+    replay()
+    replay()
+    lat.step(2)                                              # steps so far: 4 + 4 + 2
+    lat.autotune_ib([1, 3], steps_each=2)                    # 2 x (2 + 2)
+    replay()
+    l0 = lat.counters()[0]
+    lat.step(1)
+    assert lat.counters()[0] - l0 == per_step
+    _same(lat, case, prec, 21)
+    assert all(bool((j == 255).all()) for j in junk)
+    lat.close()
+
+
+def test_markers_added_after_a_capture_open_the_form_again():
+    case = wl.couette(128)
+    lat = gpu_lattice(case, "fp32")
+    _capture(lat, 2)
+    lat.step(2)
+    b = wl.couette(96).bodies[0]
+    lat.add_markers(b.xy + 16.0, b.ds, **b.as_kwargs())
+    l0 = lat.counters()[0]
+    lat.step(1)
+    assert lat.counters()[0] - l0 == 2
+    lat.close()
