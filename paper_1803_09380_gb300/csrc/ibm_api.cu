@@ -804,15 +804,17 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
       c.ev.resize(kEventsPerStep * kEventPairs);
       for (auto& e : c.ev) IBM_CK(h, cudaEventCreate(&e));
     }
+    // a captured step fixes the form; that of an unplanned lattice is the persistent kernel
+    const bool captured = c.nm > 0 && being_captured(c);
+    if (captured) c.sl_tried = c.form_fixed = true;
     if (c.nm > 0 && !c.band_valid) {
       build_band(c);
+      c.band_valid = !captured;          // the graph builds it; a plain call before its replay has to as well
       if (c.ib_phases == 1) {
         ibm_status st = count_band(h);
         if (st != IBM_OK) return st;
       }
     }
-    // a captured step fixes the form; that of an unplanned lattice is the persistent kernel
-    if (c.nm > 0 && being_captured(c)) c.sl_tried = c.form_fixed = true;
     if (c.nm > 0 && !c.sl_tried) plan_slices(c);
     const bool want_macro = !(flags & IBM_STEP_NO_MACRO);
     for (int k = 0; k < nsteps;) {

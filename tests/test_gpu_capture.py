@@ -106,3 +106,28 @@ def test_markers_added_after_a_capture_open_the_form_again():
     lat.step(1)
     assert lat.counters()[0] - l0 == 2
     lat.close()
+
+
+@pytest.mark.parametrize("planned", [False, True])
+def test_a_plain_call_before_the_first_replay_has_a_band(planned):
+    """The captured call finds no band (none yet, or a pose was written): its
+    build runs with the replays only, so a plain call ahead of them builds its
+    own."""
+    case = CASES["pair"]()
+    lat = gpu_lattice(case, "fp32")
+    if planned:
+        lat.step(2)
+        state = lat.read(ibm.FIELD_BODY_STATE)
+        state[:, 0] += 3.4
+        lat.write(ibm.FIELD_BODY_STATE, state)
+    replay = _capture(lat, 2)
+    lat.step(2)
+    replay()
+    ref = gpu_lattice(case, "fp32")
+    if planned:
+        ref.step(2)
+        ref.write(ibm.FIELD_BODY_STATE, state)
+    ref.step(4)
+    assert np.array_equal(lat.f, ref.f) and np.array_equal(lat.bodies, ref.bodies)
+    lat.close()
+    ref.close()
