@@ -253,8 +253,11 @@ void choose_ib_grid(Ctx& c) {
   // 4096^2 Couette step (14052 markers) 3/4 of the SMs gave the shortest step
   // (the correction chain still ends before collide+stream).
   const int wide = (3 * c.ib_grid_max + 3) / 4;
-  c.ib_grid = c.ib_grid_opt > 0 ? (c.ib_grid_opt < c.ib_grid_max ? c.ib_grid_opt : c.ib_grid_max)
-                                : (M <= kSmallIbMarkers ? 1 : wide);
+  // A graph that the caller captured waits at the barrier below with the grid
+  // that it was captured with: that size stays (see drop_slices).
+  if (!c.form_fixed)
+    c.ib_grid = c.ib_grid_opt > 0 ? (c.ib_grid_opt < c.ib_grid_max ? c.ib_grid_opt : c.ib_grid_max)
+                                  : (M <= kSmallIbMarkers ? 1 : wide);
   c.ib_cluster = false;
   // The grid barrier's arrival counter only grows and each barrier waits for
   // the next multiple of the grid size: a new grid size must start from a

@@ -131,3 +131,20 @@ def test_a_plain_call_before_the_first_replay_has_a_band(planned):
     assert np.array_equal(lat.f, ref.f) and np.array_equal(lat.bodies, ref.bodies)
     lat.close()
     ref.close()
+
+
+def test_the_captured_grid_of_the_persistent_kernel_stays():
+    """878 markers on 114 CTAs that wait at the barrier in global memory, whose
+    arrival counter is a multiple of the grid: another size set between the
+    replays would leave it a multiple of that one."""
+    case = wl.couette(256)
+    lat = gpu_lattice(case, "fp32")
+    ibm.ibm_set_option(lat.h, ibm.IBM_OPT_BARRIER_LIMIT_US, 200000)
+    replay = _capture(lat, 2)
+    replay()
+    lat.set_ib_ctas(95)
+    lat.step(2)
+    replay()
+    lat.step(1)
+    _same(lat, case, "fp32", 7)
+    lat.close()
