@@ -307,8 +307,12 @@ void plan_slices(Ctx& c) {
     if (c.ib_grid_opt > 1 || !slice_moving_fits(c)) return;
     c.sl_mem = dev_alloc(c, slice_mem_bytes(c.prec, 1));
     if (!c.sl_mem) return;
+    // lists that are too short for the pose at hand are so for most others of
+    // these bodies: one CTA would do the general path's work in every step
+    bool fits = false;
     if (cudaMemsetAsync(c.sl_mem, 0, slice_mem_bytes(c.prec, 1), c.stream) != cudaSuccess ||
-        launch_rebuild(c, false, c.stream) != cudaSuccess) {
+        launch_rebuild(c, false, c.stream) != cudaSuccess ||
+        slice_rebuild_fits(c, &fits, c.stream) != cudaSuccess || !fits) {
       cudaGetLastError();
       dev_free(c, c.sl_mem);
       c.sl_mem = nullptr;

@@ -345,6 +345,9 @@ int slice_max_corr();
 // band up to the bodies' pose, after moving the bodies by a step if asked.
 bool slice_moving_fits(Ctx& h);
 cudaError_t launch_rebuild(const Ctx& h, bool move, cudaStream_t s);
+// Whether the last rebuild's band fitted the slice's lists (waits for it; if
+// not, the general path's lists are complete).
+cudaError_t slice_rebuild_fits(const Ctx& h, bool* fits, cudaStream_t s);
 void launch_slice_loop(const Ctx& h, int parity, bool macro, cudaStream_t s);
 // The whole step in two launches on s (the correction, and one kernel for
 // everything else behind it); false: not on slices, or a grid too large.

@@ -1173,6 +1173,15 @@ cudaError_t launch_rebuild(const Ctx& h, bool move, cudaStream_t s) {
   return h.r_bytes == 8 ? rebuild_t<double>(h, move, s) : rebuild_t<float>(h, move, s);
 }
 
+cudaError_t slice_rebuild_fits(const Ctx& h, bool* fits, cudaStream_t s) {
+  const int* head = h.r_bytes == 8 ? slice_args<double>(h).head : slice_args<float>(h).head;
+  int flag = 0;
+  cudaError_t e = cudaMemcpyAsync(&flag, head + 3, sizeof(flag), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  *fits = e == cudaSuccess && flag == 0;
+  return e;
+}
+
 template <class R>
 static bool moving_fits_t(Ctx& h) {
   h.sl_count = 1;

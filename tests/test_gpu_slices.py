@@ -185,7 +185,7 @@ def _window_counts(xy):
     return int(grid.max()), rows
 
 
-def _plates(k):
+def _plates(k, at=((32.4, 31.3), (30.45, 29.35), (34.35, 31.4))):
     """Three plates of k x k markers two units apart in relative motion.  A node
     is covered by at most four markers of a plate; a marker couples with nine
     of its own plate and, as the window origins fall, with 9, 12 or 16 of each
@@ -193,8 +193,8 @@ def _plates(k):
     g = 2.0 * np.arange(k) - (k - 1)
     xy = np.stack(np.meshgrid(g, g), -1).reshape(-1, 2)
     bodies = []
-    for at, u in (((32.4, 31.3), (0.0, 0.0)), ((30.45, 29.35), (0.13, 0.02)), ((34.35, 31.4), (-0.03, 0.11))):
-        bodies.append(wl.Body(xy + at, np.ones(k * k), wl.BODY_PRESCRIBED, xc=at, u=u, radius=float(k)))
+    for xc, u in zip(at, ((0.0, 0.0), (0.13, 0.02), (-0.03, 0.11))):
+        bodies.append(wl.Body(xy + xc, np.ones(k * k), wl.BODY_PRESCRIBED, xc=xc, u=u, radius=float(k)))
     return wl.Case("plates", 64, 64, 0.8, bodies=bodies)
 
 
@@ -235,5 +235,36 @@ def test_moving_bodies_in_and_out_of_what_the_slice_holds(prec, make, limit):
     assert fit[0] and fit[-1] and not all(fit)
     assert np.all(np.isfinite(ref.f)) and np.array_equal(fast.f, ref.f)
     assert np.array_equal(fast.markers, ref.markers)
+    fast.close()
+    ref.close()
+
+
+# bodies on the slice (3 launches a step) and on the general path (collide+stream,
+# correction, band collide, body update, marker move, six of the band: 11)
+FORMS = {
+    "fp32 256 markers": ("fp32", lambda: _free_ring(40.0, 256), 3),
+    "fp32 257 markers": ("fp32", lambda: _free_ring(40.0, 257), 11),
+    "fp64 128 markers": ("fp64", lambda: _free_ring(20.0, 128), 3),
+    "fp64 129 markers": ("fp64", lambda: _free_ring(20.0, 129), 11),
+    # lists too short from the first pose on: five units apart (16 nodes a marker),
+    # a third of a unit apart (17 markers on a node), 41 coupled markers
+    "sparse": ("fp32", lambda: _free_ring(32.0, 40), 11),
+    "covered": ("fp32", lambda: _free_ring(11.0, 210), 11),
+    "rows": ("fp32", lambda: _plates(7, ((32.4, 31.3), (31.4, 30.3), (31.4, 32.3))), 11),
+}
+
+
+@pytest.mark.parametrize("name", sorted(FORMS))
+def test_moving_bodies_run_the_form_that_their_first_pose_fits(name):
+    prec, make, launches = FORMS[name]
+    fast, ref = gpu_lattice(make(), prec), gpu_lattice(make(), prec)
+    ibm.ibm_set_option(ref.h, ibm.IBM_OPT_IB_PHASES, 1)
+    for n in (1, 8, 2):
+        l0 = fast.counters()[0]
+        fast.step(n)
+        assert fast.counters()[0] - l0 == launches * n
+        ref.step(n)
+    assert np.array_equal(fast.f, ref.f) and np.array_equal(fast.bodies, ref.bodies)
+    assert np.array_equal(fast.resid, ref.resid) and np.array_equal(fast.markers, ref.markers)
     fast.close()
     ref.close()
