@@ -321,8 +321,11 @@ void plan_slices(Ctx& c) {
     c.sl_on = true;
     return;
   }
-  if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 8 * sizeof(int)))) return;
+  // so few CTAs that a slice's own markers are too many (a served case above 256
+  // markers by default): nothing to try
   const int asked = c.ib_grid_opt > 0 ? (c.nm + c.ib_grid - 1) / c.ib_grid : 0;
+  if (asked > kSliceMarkers) return;
+  if (!c.dslstat && !(c.dslstat = (int*)dev_alloc(c, 8 * sizeof(int)))) return;
   for (int S = asked ? asked : slice_size(c); S >= 1; S /= 2) {
     const int count = (c.nm + S - 1) / S;
     if (count > kSliceMaxCount) break;

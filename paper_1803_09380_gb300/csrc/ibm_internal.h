@@ -332,6 +332,7 @@ void launch_body_update(const Ctx& h, cudaStream_t s);
 
 // ibm_slice.cu: the barrier-free correction loop
 constexpr int kSliceMaxCount = 2048;
+constexpr int kSliceMarkers = 256;       // local markers of a slice: one per thread
 size_t slice_mem_bytes(int prec, int count);
 // Builds the lists of h.sl_count slices of h.sl_S markers into h.sl_mem;
 // stat (device, 8 ints, zeroed): a slice did not fit; largest node counts,

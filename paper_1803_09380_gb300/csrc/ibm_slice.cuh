@@ -38,7 +38,6 @@
 namespace ibm {
 
 constexpr int kSliceThreads = 256;
-constexpr int kSliceMarkers = 256;       // local markers of a slice: one per thread
 constexpr int kSliceNodes = 2048;        // local band nodes
 constexpr int kSliceX1 = 1280;           // local nodes whose second moments are formed
 constexpr int kSliceRow = 32;            // coupled markers of one marker

@@ -268,3 +268,30 @@ def test_moving_bodies_run_the_form_that_their_first_pose_fits(name):
     assert np.array_equal(fast.resid, ref.resid) and np.array_equal(fast.markers, ref.markers)
     fast.close()
     ref.close()
+
+
+@pytest.mark.parametrize("count,ctas,slices", [(256, 1, True), (257, 1, False), (513, 2, False)])
+def test_slices_too_large_to_hold_their_own_markers_are_not_tried(count, ctas, slices):
+    """As many CTAs as the per-case server pins for so many markers: above 256 a
+    CTA the first step allocates nothing and runs the persistent kernel."""
+    xy, ds = wl.ring(60.2, 59.7, count / (2 * math.pi), count=count)
+    case = wl.Case("ring", 256, 256, 0.8, bodies=[
+        wl.Body(xy + 64.0, ds, wl.BODY_FIXED, xc=(124.2, 123.7), omega=2e-4, radius=10.0)])
+    assert ibm.use_torch_allocator()
+    alloc, release = ibm._torch_hooks
+    sizes = []
+
+    def counted(nbytes, device, stream, ctx):
+        sizes.append(nbytes)
+        return alloc(nbytes, device, stream, ctx)
+    hook = ibm._ALLOC_FN(counted)
+    lat = gpu_lattice(case, "fp32")
+    lat.set_ib_ctas(ctas)
+    ibm.ibm_set_allocator(hook, release)
+    try:
+        lat.step(1)
+        lat.sync()
+    finally:
+        ibm.ibm_set_allocator(alloc, release)
+    assert bool(sizes) == slices
+    lat.close()
