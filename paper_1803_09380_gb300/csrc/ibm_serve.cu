@@ -629,6 +629,9 @@ ibm_status ibm_server_submit(ibm_server s, const ibm_case_desc* c, long long* ca
     if (c->ds) { r->ds.assign(c->ds, c->ds + M); r->has_ds = true; }
     r->bytes = case_bytes(c->lattice, M, c->nbodies);
     r->ib_ctas = server_ib_ctas(M, s->desc.ib_markers_per_cta);
+    // the slices of its correction, which the first step allocates
+    if (M > 0 && !s->desc.batched && (M + r->ib_ctas - 1) / r->ib_ctas <= ibm::kSliceMarkers)
+      r->bytes += (double)ibm::slice_mem_bytes(c->lattice.prec, r->ib_ctas);
     if (r->ib_ctas >= 2 && !s->desc.batched) {
       // a grid that cannot be scheduled as one cluster falls back to the
       // grid barrier, whose CTAs must all be resident: count those

@@ -295,3 +295,20 @@ def test_slices_too_large_to_hold_their_own_markers_are_not_tried(count, ctas, s
         ibm.ibm_set_allocator(alloc, release)
     assert bool(sizes) == slices
     lat.close()
+
+
+def test_server_counts_the_slices_in_the_memory_of_a_case():
+    """The first step of a served case allocates its slices' lists, 349 KB each
+    in FP64: 16 slices of 16 markers against one slice of 256."""
+    xy, ds = wl.ring(64.2, 63.7, 40.0, count=256)
+    case = wl.Case("ring", 128, 128, 0.8, bodies=[
+        wl.Body(xy, ds, wl.BODY_FIXED, xc=(64.2, 63.7), omega=2e-4, radius=40.0)])
+    held = []
+    for per_cta in (16, 256):
+        with ibm.Server(max_active=1, steps_per_launch=4, ib_markers_per_cta=per_cta) as srv:
+            i = srv.submit(case, 40, prec="fp64")
+            srv.progress()
+            held.append(srv.stats()["device_bytes"])
+            srv.wait(i)
+            assert srv.stats()["device_bytes"] == 0
+    assert 15 * 340e3 < held[0] - held[1] < 15 * 360e3
