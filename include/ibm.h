@@ -305,8 +305,8 @@ enum {
 };
 
 /* Chooses the correction kernel's CTA count by measurement: for each of the
- * n candidates (CTA counts as for IBM_OPT_IB_CTAS; NULL or n == 0: a default
- * set around the SM count) the lattice takes steps_each ordinary time steps,
+ * n candidates (CTA counts as for IBM_OPT_IB_CTAS; NULL or n == 0: the
+ * default choice and a set up to the SM count) the lattice takes steps_each ordinary time steps,
  * timed with CUDA events on its stream; the fastest count is then set and
  * written to *best (optional), its time per step to *best_us (optional).
  * The steps are real steps of the simulation (n * steps_each of them;

@@ -1128,10 +1128,11 @@ ibm_status ibm_autotune_ib(ibm_handle h, const int* candidates, int n, int steps
     if (candidates[k] < 0) return fail(h, IBM_ERR_INVALID, "negative candidate");
   std::vector<int> cand(candidates, candidates + n);
   if (cand.empty()) {
-    // one CTA, a cluster, and 1/2, 3/4 and all of the SMs
+    // the default choice (its slices are of a size that no CTA count gives), one
+    // CTA, a cluster, and 1/2, 3/4 and all of the SMs
     const int sms = h->ib_grid_max;
-    for (int v : {1, 8, 16, sms / 2, (3 * sms + 3) / 4, sms})
-      if (v >= 1 && std::find(cand.begin(), cand.end(), v) == cand.end()) cand.push_back(v);
+    for (int v : {0, 1, 8, 16, sms / 2, (3 * sms + 3) / 4, sms})
+      if (std::find(cand.begin(), cand.end(), v) == cand.end()) cand.push_back(v);
   }
   if (h->nm == 0) {                      // nothing to tune: no correction kernel
     if (best) *best = 0;

@@ -312,3 +312,20 @@ def test_server_counts_the_slices_in_the_memory_of_a_case():
             srv.wait(i)
             assert srv.stats()["device_bytes"] == 0
     assert 15 * 340e3 < held[0] - held[1] < 15 * 360e3
+
+
+def test_autotuner_tries_the_default_choice():
+    """The default candidates: the library's own choice of slices (0), 1, 8 and 16
+    CTAs, 1/2, 3/4 and all of the SMs, each for 2 + 4 steps."""
+    import torch
+    lat = gpu_lattice(wl.couette(96), "fp32")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    candidates = {0, 1, 8, 16, sms // 2, (3 * sms + 3) // 4, sms}
+    best, us = lat.autotune_ib(None, steps_each=4)
+    assert best in candidates and us > 0
+    assert lat.counters()[1] == 6 * len(candidates)
+    ref = gpu_lattice(wl.couette(96), "fp32")
+    ref.step(6 * len(candidates))
+    assert np.array_equal(lat.f, ref.f)
+    lat.close()
+    ref.close()
