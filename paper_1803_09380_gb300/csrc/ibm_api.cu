@@ -840,7 +840,7 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
           }
         }
         IBM_CK(h, cudaGraphLaunch(c.graph_block[parity], c.stream));
-        c.launches += (long long)kBlockSteps * kernels_per_step(c);
+        c.launches += kBlockSteps / 2 * (long long)(kernels_per_step(c, 0) + kernels_per_step(c, 1));
         c.steps += kBlockSteps;
         c.watch_due += kBlockSteps;
         watchdog_if_due(c);
@@ -867,7 +867,7 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
         IBM_CK(h, cudaGetLastError());
       }
       c.parity ^= 1;
-      c.launches += kernels_per_step(c, timing);
+      c.launches += kernels_per_step(c, parity, timing);
       c.steps += 1;
       c.watch_due += 1;
       watchdog_if_due(c);

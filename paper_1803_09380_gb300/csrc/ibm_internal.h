@@ -173,12 +173,17 @@ struct ibm_ctx : public ibm::Ctx {};
 
 namespace ibm {
 
-// Number of CUDA kernels one time step launches (matches enqueue_step; timed:
-// with the collide+stream launch bracketed).
-inline int kernels_per_step(const Ctx& h, bool timed = false) {
-  if (h.sl_on && !timed) return h.any_moving ? 3 : 2;   // correction, everything else, motion and rebuild
-  int k = 1;                                       // collide + stream
-  if (has_nee(h.geom)) k += 1;                     // extrapolation columns
+// Launches of launch_collide_stream in a step of the given parity.
+int collide_launches(const Ctx& h, int parity);
+// Whether the step behind the slices fits one launch (else the step forks).
+bool slice_step_fits(const Ctx& h);
+
+// Number of CUDA kernels that one time step launches (matches enqueue_step;
+// timed: with the collide+stream launch bracketed).
+inline int kernels_per_step(const Ctx& h, int parity, bool timed = false) {
+  if (h.sl_on && !timed && slice_step_fits(h))
+    return h.any_moving ? 3 : 2;                   // correction, everything else, motion and rebuild
+  int k = collide_launches(h, parity);
   if (h.nm > 0) {
     // correction loop (one kernel; one per phase; or pre, cluster, post),
     // band collide+stream

@@ -159,26 +159,54 @@ __global__ void k_watchdog(Geom g, const typename Prec<P>::S* __restrict__ A, in
 // ------------------------------------------------------------------ launchers
 static dim3 row_grid(const Geom& g, int bs) { return dim3((g.nx + bs - 1) / bs, g.ny); }
 
+// Grid of k_collide_stream: blocks per row and the rows of blocks that the edge
+// nodes take; beyond the grid's limit those are a launch by themselves.
+struct K1Grid {
+  int bx, edge_rows;
+  bool split;
+};
+template <int P, int PAR>
+static K1Grid k1_grid(const Geom& g) {
+  constexpr int VEC = PAR ? VecTraits<P>::VEC_ODD : VecTraits<P>::VEC;
+  const int warps_per_row = (g.nx + 32 * VEC - 1) / (32 * VEC);
+  constexpr int wpb = kK1Threads / 32;
+  K1Grid k;
+  k.bx = (warps_per_row + wpb - 1) / wpb;
+  const long long edge = PAR ? edge_nodes(g, odd_edge<VEC>(g)) : 0;
+  const long long per_row = (long long)k.bx * kK1Threads;
+  k.edge_rows = (int)((edge + per_row - 1) / per_row);
+  k.split = k.edge_rows + g.ny > 65535;
+  return k;
+}
+
+int collide_launches(const Ctx& h, int parity) {
+  bool split = false;                              // the even step has no edge rows
+  if (parity == 1) {
+    switch (h.prec) {
+      case PREC_FP64: split = k1_grid<PREC_FP64, 1>(h.geom).split; break;
+      case PREC_FP32: split = k1_grid<PREC_FP32, 1>(h.geom).split; break;
+      case PREC_FP16_DEV: split = k1_grid<PREC_FP16_DEV, 1>(h.geom).split; break;
+      default: split = k1_grid<PREC_BF16_DEV, 1>(h.geom).split; break;
+    }
+  }
+  return (split ? 2 : 1) + (has_nee(h.geom) ? 1 : 0);   // and the extrapolation columns
+}
+
 template <int P, int PAR, bool MACRO, bool MRT>
 static void launch_k1(const Ctx& h, const StepConsts<typename Prec<P>::R>& c, int mode, cudaStream_t s) {
   typedef typename Prec<P>::S S;
   typedef typename Prec<P>::R R;
   S* A = (S*)h.f;
   R* mac = (R*)h.macro;
-  constexpr int VEC = PAR ? VecTraits<P>::VEC_ODD : VecTraits<P>::VEC;
-  const int warps_per_row = (h.geom.nx + 32 * VEC - 1) / (32 * VEC);
-  constexpr int wpb = kK1Threads / 32;
-  const int bx = (warps_per_row + wpb - 1) / wpb;
-  const long long edge = PAR ? edge_nodes(h.geom, odd_edge<VEC>(h.geom)) : 0;
-  const long long per_row = (long long)bx * kK1Threads;
-  const int edge_rows = (int)((edge + per_row - 1) / per_row);
+  const K1Grid k = k1_grid<P, PAR>(h.geom);
   auto kern = mode == K1_MAIN ? k_collide_stream<P, PAR, MACRO, K1_MAIN, MRT>
                               : k_collide_stream<P, PAR, MACRO, K1_ALL, MRT>;
-  if (edge_rows + h.geom.ny <= 65535) {
-    kern<<<dim3(bx, edge_rows + h.geom.ny), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, edge_rows);
-  } else {                                    // beyond the grid's limit: the edge nodes by themselves
-    kern<<<dim3(bx, edge_rows), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, edge_rows);
-    kern<<<dim3(bx, h.geom.ny), kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, 0);
+  const dim3 all(k.bx, k.edge_rows + h.geom.ny), edges(k.bx, k.edge_rows), rows(k.bx, h.geom.ny);
+  if (!k.split) {
+    kern<<<all, kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, k.edge_rows);
+  } else {
+    kern<<<edges, kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, k.edge_rows);
+    kern<<<rows, kK1Threads, 0, s>>>(h.geom, c, A, mac, h.dsegflag, h.nseg_x, 0);
   }
 }
 

@@ -1341,6 +1341,18 @@ static StepShape step_shape(const Ctx& h, bool fprev, bool fnow) {
 }
 static long long step_rows(const StepShape& sh) { return (long long)sh.edge_rows + sh.span_rows + sh.tail_rows; }
 
+// The same answer for every step of the lattice.
+template <int P>
+static bool step_fits_t(const Ctx& h) { return step_rows(step_shape<P, 1>(h, true, true)) <= 65535; }
+bool slice_step_fits(const Ctx& h) {
+  switch (h.prec) {
+    case PREC_FP64: return step_fits_t<PREC_FP64>(h);
+    case PREC_FP32: return step_fits_t<PREC_FP32>(h);
+    case PREC_FP16_DEV: return step_fits_t<PREC_FP16_DEV>(h);
+    default: return step_fits_t<PREC_BF16_DEV>(h);
+  }
+}
+
 template <int P, int PAR, bool MACRO, bool MRT>
 static void launch_stream(const Ctx& h, cudaStream_t s, const IbArgs<P>& a,
                           const SliceArgs<typename Prec<P>::R>& sl, bool fprev, bool fnow) {
@@ -1359,8 +1371,7 @@ static void launch_stream(const Ctx& h, cudaStream_t s, const IbArgs<P>& a,
 
 template <int P>
 static bool slice_step_t(const Ctx& h, int parity, bool macro, bool fprev, bool fnow, cudaStream_t s) {
-  // the same answer for every step of the lattice
-  if (step_rows(step_shape<P, 1>(h, true, true)) > 65535) return false;
+  if (!step_fits_t<P>(h)) return false;
   IbArgs<P> a = make_ib_args<P>(h);
   SliceArgs<typename Prec<P>::R> sl = slice_args<typename Prec<P>::R>(h);
   launch_slices<P>(h, parity, s, a, sl);

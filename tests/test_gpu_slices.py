@@ -329,3 +329,27 @@ def test_autotuner_tries_the_default_choice():
     assert np.array_equal(lat.f, ref.f)
     lat.close()
     ref.close()
+
+
+def test_launches_are_counted_where_a_step_does_not_fit_one_grid():
+    """16 x 65535 nodes between walls: edge rows and lattice rows of the odd step
+    go as two launches, and with markers the step forks (slices, band segments,
+    collide+stream)."""
+    def make(bodies):
+        return wl.Case("tall", 16, 65535, 0.8, bc=(wl.BOUNCEBACK,) * 4, wall_u=(0,) * 6 + (0.03, 0), bodies=bodies)
+    xy, ds = wl.ring(7.6, 65520.3, 4.0, count=25)
+    ring = wl.Body(xy, ds, wl.BODY_FIXED, xc=(7.6, 65520.3), omega=1e-3, radius=4.0)
+    for bodies, even, odd in (([], 1, 2), ([ring], 3, 4)):
+        out = []
+        for phases in (0, 1):
+            lat = gpu_lattice(make(bodies), "fp32")
+            ibm.ibm_set_option(lat.h, ibm.IBM_OPT_IB_PHASES, phases)
+            for n, want in ((1, even), (1, odd), (9, 5 * even + 4 * odd)):
+                l0 = lat.counters()[0]
+                lat.step(n)
+                if not phases:
+                    assert lat.counters()[0] - l0 == want
+            out.append((lat.f, lat.bodies, lat.resid))
+            lat.close()
+        for a, b in zip(*out):
+            assert np.all(np.isfinite(a)) and np.array_equal(a, b)
