@@ -38,6 +38,15 @@ struct DeviceGuard {
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
+// Allocating on a step's behalf must not end a capture that this or another
+// thread has under way on another stream: the stricter modes forbid that to
+// every thread that has not asked for the relaxed one.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // In pool mode every allocation of at most kPoolCarveMax bytes is carved from
 // a kPoolChunk chunk of the pool, released with the lattice.  Each call to the
 // pool's allocator costs host time (about 0.4 ms per call was measured once
@@ -299,6 +308,7 @@ void plan_slices(Ctx& c) {
     cudaGetLastError();
     return;
   }
+  RelaxedCapture relaxed;
   c.sl_tried = true;
   if (c.nm == 0 || !c.band_collide || c.ib_phases != 0 || c.ib_threads != kIbThreads ||
       c.test_drop_arrival || c.desc.n_corr < 1 || c.desc.n_corr > slice_max_corr())

@@ -148,3 +148,38 @@ def test_the_captured_grid_of_the_persistent_kernel_stays():
     lat.step(1)
     _same(lat, case, "fp32", 7)
     lat.close()
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_first_steps_while_another_stream_is_captured(name):
+    """The slices' lists are allocated by the first steps, here with cudaMalloc
+    while the caller captures another stream in the strictest mode: neither
+    the steps nor the capture fail."""
+    import torch
+    case = CASES[name]()
+    alloc, release = ibm._torch_hooks if ibm.use_torch_allocator() else (None, None)
+    x = torch.zeros(1000, device="cuda")
+    side = torch.cuda.Stream()
+    ref = gpu_lattice(case, "fp32")
+    ref.step(5)
+    want = (ref.f, ref.bodies)
+    ref.close()
+    ibm.ibm_set_allocator(None, None)
+    try:
+        lat = ibm.Lattice(case.nx, case.ny, case.tau, case.rho0, "fp32", case.bc, case.wall_u, case.inlet_u,
+                          case.n_corr, torch_stream=False)
+        for b in case.bodies:
+            lat.add_markers(b.xy, b.ds, **b.as_kwargs())
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side, capture_error_mode="global"):
+            x += 1
+            lat.step(2, ibm.STEP_NO_GRAPH)
+            x += 1
+        g.replay()
+        lat.step(3)
+        assert np.array_equal(lat.f, want[0]) and np.array_equal(lat.bodies, want[1])
+        lat.close()
+    finally:
+        ibm.ibm_set_allocator(alloc, release)
+    torch.cuda.synchronize()
+    assert bool((x == 2).all())
