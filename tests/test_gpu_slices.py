@@ -314,19 +314,21 @@ def test_server_counts_the_slices_in_the_memory_of_a_case():
     assert 15 * 340e3 < held[0] - held[1] < 15 * 360e3
 
 
-def test_autotuner_tries_the_default_choice():
+@pytest.mark.parametrize("name", ["couette", "pair"])
+def test_autotuner_tries_the_default_choice(name):
     """The default candidates: the library's own choice of slices (0), 1, 8 and 16
     CTAs, 1/2, 3/4 and all of the SMs, each for 2 + 4 steps."""
     import torch
-    lat = gpu_lattice(wl.couette(96), "fp32")
+    make = (lambda: wl.couette(96)) if name == "couette" else MOVING["pair"]
+    lat = gpu_lattice(make(), "fp32")
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     candidates = {0, 1, 8, 16, sms // 2, (3 * sms + 3) // 4, sms}
     best, us = lat.autotune_ib(None, steps_each=4)
     assert best in candidates and us > 0
     assert lat.counters()[1] == 6 * len(candidates)
-    ref = gpu_lattice(wl.couette(96), "fp32")
+    ref = gpu_lattice(make(), "fp32")
     ref.step(6 * len(candidates))
-    assert np.array_equal(lat.f, ref.f)
+    assert np.array_equal(lat.f, ref.f) and np.array_equal(lat.bodies, ref.bodies)
     lat.close()
     ref.close()
 
@@ -353,3 +355,21 @@ def test_launches_are_counted_where_a_step_does_not_fit_one_grid():
             lat.close()
         for a, b in zip(*out):
             assert np.all(np.isfinite(a)) and np.array_equal(a, b)
+
+
+def _launches(lat):
+    l0 = lat.counters()[0]
+    lat.step(2)
+    return (lat.counters()[0] - l0) // 2
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16", "bf16"])
+def test_the_cases_above_run_on_slices(prec):
+    """What is compared with the phase kernels above is the slices: two launches a
+    step with fixed markers, three with moving ones.  FP64 holds 128 moving
+    markers: the three cases with more run the general path."""
+    for name in sorted(CASES):
+        assert _launches(gpu_lattice(CASES[name](), prec)) == 2, name
+    for name in sorted(MOVING):
+        general = prec == "fp64" and name in ("mixed", "most", "dense")
+        assert _launches(gpu_lattice(MOVING[name](), prec)) == (11 if general else 3), name
