@@ -824,9 +824,11 @@ ibm_status ibm_step(ibm_handle h, int nsteps, unsigned flags) {
       c.ev.resize(kEventsPerStep * kEventPairs);
       for (auto& e : c.ev) IBM_CK(h, cudaEventCreate(&e));
     }
-    // a captured step fixes the form; that of an unplanned lattice is the persistent kernel
-    const bool captured = c.nm > 0 && being_captured(c);
-    if (captured) c.sl_tried = c.form_fixed = true;
+    // a captured step fixes the form; that of an unplanned lattice is the persistent
+    // kernel (replays of the library's own graphs, which no capture admits, do not ask)
+    const bool captured =
+        c.nm > 0 && (!use_graph || !c.sl_tried || !c.band_valid) && being_captured(c);
+    if (captured && !use_graph) c.sl_tried = c.form_fixed = true;
     if (c.nm > 0 && !c.band_valid) {
       build_band(c);
       c.band_valid = !captured;          // the graph builds it; a plain call before its replay has to as well
