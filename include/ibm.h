@@ -267,14 +267,21 @@ enum {
   IBM_OPT_IB_CTAS = 1,  /* CTAs of the correction kernel; n > 0 = min(n, SMs).  Markers that keep
                            their places are dealt to the CTAs in slices, each iterated with
                            the neighbourhood it depends on, without a barrier (0, the default:
-                           a slice per SM, of 4 (FP64) or 8 to 128 markers); up to 256 markers of
-                           moving bodies run on one CTA.  Where the slices do not fit (too few
-                           CTAs for the markers, very dense markers, more than 60 iterations)
-                           a persistent kernel with a grid barrier runs instead: 0 = one CTA
-                           for up to 512 markers, 3 per 4 SMs above that; 2..16 CTAs run as
-                           one thread-block cluster when the device can schedule it.  Results
-                           do not depend on it. */
-  IBM_OPT_IB_THREADS = 2, /* threads per correction-kernel CTA: 256 (default), 512 or 1024 */
+                           a slice per SM, of 4 (FP64) or 8 to 128 markers).  Moving bodies run on
+                           one CTA (n <= 1) whose lists are rebuilt every step: up to 256
+                           markers at up to 10 iterations, 192 at 25, 118 at 60; in FP64 128, 96
+                           and 64; if their first pose fits the lists (8 to 12 markers on a
+                           node, 32 coupled with one, 7 nodes a marker and 32 to 63 more; a ring
+                           of markers a lattice unit apart needs 6, 10 and 5).  The lists
+                           take 218 KB of device memory a slice, 349 KB in FP64.  Where the
+                           slices do not fit (too few CTAs for the markers, very dense or
+                           sparse markers, more than 60 iterations, no memory) a persistent
+                           kernel with a grid barrier runs instead: 0 = one CTA for up to 512
+                           markers, 3 per 4 SMs above that; 2..16 CTAs run as one thread-block
+                           cluster when the device can schedule it.  Results do not depend on
+                           it. */
+  IBM_OPT_IB_THREADS = 2, /* threads per correction-kernel CTA: 256 (default); 512 or 1024 select
+                           the persistent kernel */
   IBM_OPT_WATCHDOG_STEPS = 3, /* K > 0: after every K steps (at the next 8-step block boundary)
                            scan every stored population for NaN/Inf; a hit makes the next
                            synchronising call return IBM_ERR_DIVERGED.  0 (default): no scan.

@@ -297,11 +297,14 @@ int slice_size(const Ctx& c) {
 }
 
 // Plans the barrier-free correction for the current band: builds the slices'
-// lists, halving the slices while one does not fit; moving bodies of up to 256
-// markers run on one slice that is rebuilt every step.  Without it (more
-// moving markers, another launch form asked for, markers too dense for any slice, no
-// memory) steps run the persistent kernel.  Synchronises the stream once
-// per attempt; a stream that is being captured is left alone.
+// lists, halving the slices while one does not fit; moving bodies run on one
+// slice that is rebuilt every step, where their markers fit its shared memory (at
+// 10 iterations 256 with FP32 arithmetic, 128 in FP64) and their first pose its
+// lists.  Without it (more moving markers, another launch form asked for, markers
+// too dense for any slice, no memory) steps run the persistent kernel.
+// Synchronises the stream once per attempt; a stream that is being captured is
+// left alone.  The lists take 218 KB a slice (349 KB in FP64), whatever it holds:
+// their strides are those of the largest slice.
 void plan_slices(Ctx& c) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -435,9 +438,9 @@ ibm_status upload_markers(Ctx* h) {
   IBM_ALLOC(h, c.dbcnt, int*, c.bcap);
   c.dent = dev_alloc(c, (R == 8 ? sizeof(Ent<double>) : sizeof(Ent<float>)) * (size_t)c.bcap * kBandCap);
   IBM_ALLOC(h, c.dfpart, double*, (size_t)((M + kForceChunk - 1) / kForceChunk) * c.nb * 3 * 2);
-  // correction-kernel CTAs: one for small boundaries (its grid barrier is a
-  // block barrier, so such kernels of several lattices may run side by
-  // side), one per SM otherwise
+  // persistent-kernel CTAs: one for small boundaries (its grid barrier is a block
+  // barrier, so such kernels of several lattices may run side by side), three
+  // per four SMs otherwise
   choose_ib_grid(c);
   c.dbq = dev_alloc(c, R * 8 * (size_t)c.bcap);
   c.dmq = dev_alloc(c, R * 4 * (size_t)M);

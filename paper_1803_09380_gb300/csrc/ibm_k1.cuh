@@ -502,8 +502,8 @@ constexpr int k1_min_blocks(int P, int PAR) {
 // thread through the boundary rules, in blocks (or thread strides) of their
 // own: beside the vector path they cost it registers, and whole spans of them,
 // four nodes in turn per lane, made the odd step of a 1600 x 800 FP32 channel
-// 46.5 us against 13.9 for the even one (now 22.2; a 1001 x 777 closed box in
-// FP16 storage 16.4 -> 8.2 us a step).
+// 46.5 us against 13.9 for the even one (now 16.4 to 17.0 beside 12.6 to 13.8; a
+// 1001 x 777 closed box in FP16 storage 16.4 -> 6.5 us a step).
 struct OddEdge {
   int wall_rows;       // 1: rows 0 and ny - 1 are closed
   int left, right;     // vectors at x0 < left or x0 >= right are edge nodes

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_slice_build(SliceArgs<R> sl, 
 // rho and j of U band nodes at once: their 9 U loads are in flight together.
 // Away from the sides (and in the even step everywhere) the locations are
 // constant offsets; false: some node needs the boundary rules instead.
-template <int P, int PAR>
+template <int PAR>
 __device__ __forceinline__ bool plain_node(const Geom& g, int x, int y) {
   return PAR == 0 || (x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1);
 }
@@ -199,7 +199,7 @@ __device__ __forceinline__ bool gather_nodes(const IbArgs<P>& a, const int (&n)[
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int y = n[u] / g.nx, x = n[u] - y * g.nx;
-    const bool plain = plain_node<P, PAR>(g, x, y);
+    const bool plain = plain_node<PAR>(g, x, y);
     all = all && plain;
     const long long base = (long long)y * g.nxp + x;
 #pragma unroll
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) k_ib_slice(IbArgs<P> a, Slic
 #pragma unroll 1
       for (int k = t; k < nX; k += NT) {
         const int n = nid[k], y = n / a.g.nx, x = n - y * a.g.nx;
-        if (plain_node<P, PAR>(a.g, x, y)) continue;
+        if (plain_node<PAR>(a.g, x, y)) continue;
         R p[9];
         post_stream9<P>(a.g, a.c, a.A, PAR, x, y, p);
         moments9<R>(p, nr[k], njx[k], njy[k]);
@@ -761,12 +761,12 @@ __global__ void __launch_bounds__(kFinishThreads) k_band_finish(IbArgs<P> a, Sli
 // (odd step), the band-free spans and the extrapolation columns, which need
 // nothing of the correction and run beside it, then the band segments, which
 // wait for it.  Those come after three quarters of the lattice's rows: on a
-// large lattice they then find the correction done (20 us into the 175 to 190
-// us of a 4096^2 FP32 step) instead of holding registers while they wait, and
-// are not the launch's tail, where their dependent loads took 10 us.  The
-// correction releases this launch at its start: released after its gather, it
-// ended earlier (17 against 21 us) but the step later (188 and 204 us, even
-// and odd, against 185 and 201).  One stream and two launches a step, without
+// large lattice they then find the correction done (20 to 23 us into the 185 and
+// 201 us, even and odd, of a 4096^2 FP32 step) instead of holding registers while
+// they wait, and are not the launch's tail, where their dependent loads took 10
+// us.  The correction releases this launch at its start: released after its
+// gather, it ended earlier (17 against 21 us) but the step later (188 and 204 us
+// against 185 and 201).  One stream and two launches a step, without
 // fork, join or priorities.
 //
 // The forces are the longest chain behind the correction (5 us against 1.5
@@ -845,7 +845,7 @@ constexpr int kRebuildThreads = 1024;
 template <class R>
 struct RebuildArgs {
   Geom g;
-  int M, nb, N, points, nseg_x, bcap, segcap, move;
+  int M, nb, points, nseg_x, bcap, segcap, move;
   int xcap, ecap;                  // nodes and covering markers that the lists hold
   BodyDev* bodies;
   const int* mbody;
@@ -1135,7 +1135,6 @@ static cudaError_t rebuild_t(const Ctx& h, bool move, cudaStream_t s) {
   a.g = h.geom;
   a.M = h.nm;
   a.nb = h.nb;
-  a.N = h.desc.n_corr;
   a.points = h.desc.delta_points;
   a.nseg_x = h.nseg_x;
   a.bcap = h.bcap;
